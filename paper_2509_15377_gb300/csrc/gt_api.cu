@@ -919,6 +919,7 @@ static int plan_run(gt_ctx *ctx, const gt_run *r, const gt_endpoints *o, void *w
     p.status = o->status; p.aval = o->aval; p.uid = o->uid; p.nflight = o->n_flight;
     p.tallies = o->tallies; p.electrons = o->electrons;
     p.capacity = o->capacity;
+    p.n_primaries = np;
     p.hdr = reinterpret_cast<Header *>(base + Ly.hdr);
     p.ready = reinterpret_cast<unsigned int *>(base + Ly.ready);
     p.bvx = reinterpret_cast<double *>(base + Ly.bvx);

@@ -128,6 +128,7 @@ struct RunParams {
     uint64_t *tallies;    // [n_avalanches][n_levels + 1]
     uint64_t *electrons;  // [n_avalanches]
     int64_t capacity;
+    int64_t n_primaries;  // slots below are primaries, the others new electrons
     // work space
     Header *hdr;
     unsigned int *ready;      // [capacity] queue slot filled
