@@ -797,6 +797,21 @@ static int field_setup_impl(gt_ctx *ctx, const gt_field *f)
         d.box_lo_f[i] = (float)(d.origin[i] + m);
         d.box_hi_f[i] = (float)(d.hi[i] - m);
     }
+    if (d.has_b) {
+        const double w2 = d.w[0] * d.w[0] + d.w[1] * d.w[1] + d.w[2] * d.w[2];
+        d.w_abs = std::sqrt(w2);
+        d.inv_w = 1.0 / d.w_abs;
+        d.inv_w2 = 1.0 / w2;
+        const float *wf = d.w_f;
+        d.w2_f = std::fmaf(wf[2], wf[2], std::fmaf(wf[0], wf[0], wf[1] * wf[1]));
+        d.w_abs_f = std::sqrt(d.w2_f);
+        d.inv_w_f = 1.0f / d.w_abs_f;
+        d.inv_w2_f = 1.0f / d.w2_f;
+        for (int i = 0; i < 3; ++i) {
+            d.w_dir[i] = d.w[i] / d.w_abs;
+            d.w_dir_f[i] = wf[i] / d.w_abs_f;
+        }
+    }
     d.cell_hi_f[0] = (float)(d.nx - 2); d.cell_hi_f[1] = (float)(d.ny - 2);
     d.cell_hi_f[2] = (float)(d.nz - 2);
     d.node_hi_f[0] = (float)(d.nx - 1); d.node_hi_f[1] = (float)(d.ny - 1);
