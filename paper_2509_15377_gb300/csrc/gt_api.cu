@@ -1040,10 +1040,21 @@ static int plan_run(gt_ctx *ctx, const gt_run *r, const gt_endpoints *o, void *w
     pl.smem = smem;
     pl.fp64 = fp64;
     pl.smem_table = smem_table;
+    p.cell_off = 0;
     if (r->mode == GT_BATCHED) {
         const int occ = fp64 ? occupancy_batched_fp64(ctx->field.kind, block, smem)
                              : occupancy_batched_mixed(ctx->field.kind, smem_table, block, smem);
         if (occ < 1) return GT_ERR_UNSUPPORTED;
+        // mesh, mixed precision: the threads' elements in shared memory where
+        // they fit beside the rest without a CTA less per SM
+        if (!fp64 && ctx->field.kind == GT_FIELD_MESH) {
+            const size_t with = align16(smem) + (size_t)kMeshRows * block * sizeof(float4);
+            if (with <= smem_cap &&
+                occupancy_batched_mixed(GT_FIELD_MESH, smem_table, block, with) == occ) {
+                p.cell_off = (int)align16(smem);
+                pl.smem = with;
+            }
+        }
         pl.grid = r->grid ? r->grid : ctx->sms * occ;
     }
     return GT_OK;

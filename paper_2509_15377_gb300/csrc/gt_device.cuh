@@ -147,6 +147,8 @@ struct RunParams {
     int majorant;           // GT_MAJORANT_GLOBAL / GT_MAJORANT_BANDED
     double window;          // banded: window factor c
     float window_f;
+    int cell_off;           // MESH mixed: byte offset of the threads' elements in dynamic
+                            // shared memory (0: none)
     int substeps;           // field evaluations per flight (1: held field)
     int crossing;           // 1: leaving electrons end at the first crossing
     int signal_kind;        // readout electrode (GT_W_*), GT_W_NONE: no signal
@@ -363,32 +365,45 @@ __device__ __forceinline__ int mesh_find64(const DevField &f, double x, double y
 }
 
 // Walk from element t towards r (FP32): while r is not inside with every
-// coordinate >= tol (margin units), step across the face opposite the node
+// coordinate >= the element's margin, step across the face opposite the node
 // of the most negative coordinate; -1 when the walk leaves the mesh or takes
-// more than kMeshWalk steps (the bins decide then).
+// more than kMeshWalk steps (the bins decide then), -2 when r lies within the
+// margins of one face: both elements of the face see it within their margin
+// of that face and beyond their margin of every other, so that one of the two
+// holds it, FP32 cannot tell which, and no other element passes the bins'
+// test either.  (Walking on goes back and forth between the two, and the
+// bins' scan reads every element of a bin, ~250 near the wire of a graded
+// mesh: the 48-avalanche mesh run 52 -> 49.7 ms.)
+// v, m0, m1, m2 are the first rows of t's record.
 constexpr int kMeshWalk = 8;
 
 __device__ __forceinline__ int mesh_walk32(const DevField &f, float x, float y, float z, int t,
-                                           float tol)
+                                           float4 v, float4 m0, float4 m1, float4 m2)
 {
-    for (int step = 0; step < kMeshWalk; ++step) {
-        const float4 *q = f.tet32 + (kMeshRec / 4) * (int64_t)t;
-        const float4 v = __ldg(q), m0 = __ldg(q + 1), m1 = __ldg(q + 2), m2 = __ldg(q + 3);
+    int from = -1;  // the element across the face, when r is undecided there
+    for (int step = 0;; ++step) {
         const float dx = x - v.x, dy = y - v.y, dz = z - v.z;
         const float l1 = fmaf(m0.x, dx, fmaf(m0.y, dy, m0.z * dz));
         const float l2 = fmaf(m1.x, dx, fmaf(m1.y, dy, m1.z * dz));
         const float l3 = fmaf(m2.x, dx, fmaf(m2.y, dy, m2.z * dz));
-        float mn = 1.0f - l1 - l2 - l3;
+        const float l0 = 1.0f - l1 - l2 - l3;
+        float mn = l0;
         int im = 0;
         if (l1 < mn) { mn = l1; im = 1; }
         if (l2 < mn) { mn = l2; im = 2; }
         if (l3 < mn) { mn = l3; im = 3; }
-        if (mn >= tol * v.w) return t;
+        if (mn >= v.w) return t;
+        if (step == kMeshWalk - 1) return -1;
+        const bool one = mn > -v.w && (l0 < v.w) + (l1 < v.w) + (l2 < v.w) + (l3 < v.w) == 1;
         const int4 nb = __ldg(f.tet_nb + t);
-        t = im == 0 ? nb.x : im == 1 ? nb.y : im == 2 ? nb.z : nb.w;
-        if (t < 0) return -1;
+        const int next = im == 0 ? nb.x : im == 1 ? nb.y : im == 2 ? nb.z : nb.w;
+        if (next < 0) return -1;
+        if (one && next == from) return -2;
+        from = one ? t : -1;
+        t = next;
+        const float4 *q = f.tet32 + (kMeshRec / 4) * (int64_t)t;
+        v = __ldg(q); m0 = __ldg(q + 1); m1 = __ldg(q + 2); m2 = __ldg(q + 3);
     }
-    return -1;
 }
 
 // The FP64 search (closed elements) of the position r = (x, y, z), which is
@@ -419,16 +434,25 @@ __device__ __forceinline__ int mesh_find_mixed(const DevField &f, double x, doub
     return -1;
 }
 
-// Field of element record q at r (linear interpolation of the nodal values).
+// Linear interpolation of an element's nodal values at r: node v, value
+// (e0, e1, e2) there, gradient rows gx, gy, gz.
+__device__ __forceinline__ void mesh_linear32(float4 v, float e0, float e1, float e2, float4 gx,
+                                              float4 gy, float4 gz, float x, float y, float z,
+                                              float &ex, float &ey, float &ez)
+{
+    const float dx = x - v.x, dy = y - v.y, dz = z - v.z;
+    ex = fmaf(gx.x, dx, fmaf(gx.y, dy, fmaf(gx.z, dz, e0)));
+    ey = fmaf(gy.x, dx, fmaf(gy.y, dy, fmaf(gy.z, dz, e1)));
+    ez = fmaf(gz.x, dx, fmaf(gz.y, dy, fmaf(gz.z, dz, e2)));
+}
+
+// Field of element record q at r.
 __device__ __forceinline__ void mesh_field32(const float4 *q, float x, float y, float z, float &ex,
                                              float &ey, float &ez)
 {
-    const float4 v = __ldg(q), e = __ldg(q + 4), gx = __ldg(q + 5), gy = __ldg(q + 6),
-                 gz = __ldg(q + 7);
-    const float dx = x - v.x, dy = y - v.y, dz = z - v.z;
-    ex = fmaf(gx.x, dx, fmaf(gx.y, dy, fmaf(gx.z, dz, e.x)));
-    ey = fmaf(gy.x, dx, fmaf(gy.y, dy, fmaf(gy.z, dz, e.y)));
-    ez = fmaf(gz.x, dx, fmaf(gz.y, dy, fmaf(gz.z, dz, e.z)));
+    const float4 e = __ldg(q + 4);
+    mesh_linear32(__ldg(q), e.x, e.y, e.z, __ldg(q + 5), __ldg(q + 6), __ldg(q + 7), x, y, z, ex,
+                  ey, ez);
 }
 
 // Field (c = 0..2) or weighting potential (c = 3) of FP64 element record q at r.
@@ -438,6 +462,39 @@ __device__ __forceinline__ double mesh_value64(const double *q, int c, double x,
     if (c == 3) return q[19] + q[23] * dx + q[27] * dy + q[31] * dz;
     const double *g = q + 20 + 4 * c;
     return q[16 + c] + g[0] * dx + g[1] * dy + g[2] * dz;
+}
+
+// ---------------------------------------- the thread's element (mixed step)
+// A flight is much shorter than an element (about 0.1 um against 1.4-12 um),
+// so most flights start and end in the element of the one before.  Each
+// thread keeps the 25 values of its element's record that a flight uses in
+// shared memory (rows of float4 [row][thread]: no bank conflicts) and reads
+// the record itself only when it enters another: the nine scattered 16-byte
+// loads of every flight came from L2 (48-avalanche mesh run 49.7 -> 45.2 ms;
+// the same for a regular grid's eight nodes gained nothing, 110 -> 114 ms).
+constexpr int kMeshRows = 7;
+
+// The thread's element, row i at [i * blockDim.x].
+__device__ __forceinline__ float4 *cell_slot(const RunParams &p)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    return reinterpret_cast<float4 *>(smem + p.cell_off) + threadIdx.x;
+}
+
+// Keeps element t's record: v0 and margin; the rows of M,
+// each with a component of E(v0); the rows of the field's gradient.
+__device__ __forceinline__ void mesh_keep(const RunParams &p, int t)
+{
+    const float4 *q = p.field.tet32 + (kMeshRec / 4) * (int64_t)t;
+    float4 *c = cell_slot(p);
+    const unsigned S = blockDim.x;
+    const float4 v = __ldg(q), m0 = __ldg(q + 1), m1 = __ldg(q + 2), m2 = __ldg(q + 3),
+                 e = __ldg(q + 4), gx = __ldg(q + 5), gy = __ldg(q + 6), gz = __ldg(q + 7);
+    c[0] = v;
+    c[S] = make_float4(m0.x, m0.y, m0.z, e.x);
+    c[2 * S] = make_float4(m1.x, m1.y, m1.z, e.y);
+    c[3 * S] = make_float4(m2.x, m2.y, m2.z, e.z);
+    c[4 * S] = gx; c[5 * S] = gy; c[6 * S] = gz;
 }
 
 // --------------------------------------------------------------- fields
@@ -1485,6 +1542,13 @@ struct MixedElectron {
 
     __device__ __forceinline__ void bind(const Tables &tb) { b = tb.base + threadIdx.x; }
 
+    // MESH: the position's element is t from now on.
+    __device__ __forceinline__ void enter(const RunParams &p, int t)
+    {
+        if (t != elem && t >= 0 && p.cell_off) mesh_keep(p, t);
+        elem = t;
+    }
+
     // Field at the current position.  On a mesh, the element found by the
     // last boundary test holds the position (searched once for a new electron).
     template <int FK>
@@ -1492,14 +1556,21 @@ struct MixedElectron {
     {
         if (FK == GT_FIELD_MESH) {
             const float x = px + ox, y = py + oy, z = pz + oz;
-            if (elem < 0) elem = mesh_find32(p.field, x, y, z, -1, -1.0f);
+            if (elem < 0) enter(p, mesh_find32(p.field, x, y, z, -1, -1.0f));
             if (elem < 0) {  // the FP32 position's bin missed: search in FP64
                 const unsigned S = blockDim.x;
-                elem = mesh_find64(p.field, b[0] + (double)ox, b[S] + (double)oy,
-                                   b[2 * S] + (double)oz, -1, 0.0);
+                enter(p, mesh_find64(p.field, b[0] + (double)ox, b[S] + (double)oy,
+                                     b[2 * S] + (double)oz, -1, 0.0));
             }
             if (elem < 0) {
                 ex = ey = ez = 0.f;
+                return;
+            }
+            if (p.cell_off) {
+                const float4 *c = cell_slot(p);
+                const unsigned S = blockDim.x;
+                mesh_linear32(c[0], c[S].w, c[2 * S].w, c[3 * S].w, c[4 * S], c[5 * S], c[6 * S], x,
+                              y, z, ex, ey, ez);
                 return;
             }
             mesh_field32(p.field.tet32 + (kMeshRec / 4) * (int64_t)elem, x, y, z, ex, ey, ez);
@@ -1625,7 +1696,8 @@ struct MixedElectron {
         nf = nreal = nnull = n0 = 0;
         status = 0;
         timed = false;
-        elem = FK == GT_FIELD_MESH ? p.belem[s] : -1;
+        elem = -1;
+        if (FK == GT_FIELD_MESH) enter(p, p.belem[s]);
         set_base<FK>(p, p.x0[s], p.y0[s], p.z0[s], p.t0[s]);
         if (GEO) signal_start(p);
     }
@@ -1653,10 +1725,23 @@ struct MixedElectron {
                               (rx > f.box_hi_f[0]) || (ry < f.box_lo_f[1]) ||
                               (ry > f.box_hi_f[1]) || (rz < f.box_lo_f[2]) || (rz > f.box_hi_f[2]);
             if (!near) {
-                int t = elem >= 0 ? mesh_walk32(f, rx, ry, rz, elem, 1.0f) : -1;
-                if (t < 0) t = mesh_find32(f, rx, ry, rz, -1, 1.0f);
+                int t = -1;
+                if (elem >= 0) {
+                    // the element's first rows, as kept or from the record
+                    float4 v, m0, m1, m2;
+                    if (p.cell_off) {
+                        const float4 *c = cell_slot(p);
+                        const unsigned S = blockDim.x;
+                        v = c[0]; m0 = c[S]; m1 = c[2 * S]; m2 = c[3 * S];
+                    } else {
+                        const float4 *q = f.tet32 + (kMeshRec / 4) * (int64_t)elem;
+                        v = __ldg(q); m0 = __ldg(q + 1); m1 = __ldg(q + 2); m2 = __ldg(q + 3);
+                    }
+                    t = mesh_walk32(f, rx, ry, rz, elem, v, m0, m1, m2);
+                }
+                if (t == -1) t = mesh_find32(f, rx, ry, rz, -1, 1.0f);
                 if (t >= 0) {
-                    elem = t;
+                    enter(p, t);
                     return 0;
                 }
             }
@@ -1665,7 +1750,7 @@ struct MixedElectron {
             if (f.wire_r2 > 0.0 && x * x + y * y <= f.wire_r2) return GT_ST_WIRE;
             const int t = mesh_find_mixed(f, x, y, z, rx, ry, rz, elem);
             if (t < 0) return GT_ST_OUT_OF_MAP;
-            elem = t;
+            enter(p, t);
             return 0;
         } else if (FK == GT_FIELD_PLATE) {
             maybe = (oz >= zhi) || (oz < zlo);
