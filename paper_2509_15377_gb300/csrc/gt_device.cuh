@@ -963,10 +963,10 @@ __device__ __forceinline__ double scatter64(double xi, double vx, double vy, dou
 __device__ __forceinline__ float scatter32(float xi, float vx, float vy, float vz, float u, float w,
                                            float &nx, float &ny, float &nz)
 {
-    const float den = fmaf(-2.0f * xi, u, 1.0f + xi);
-    const float mu = __fdividef(fmaf(-2.0f, u, 1.0f + xi), den);
-    const float om = __fdividef(2.0f * u * (1.0f - xi), den);
-    const float sc = sqrtf(fmaxf(om * (2.0f - om), 0.0f));
+    const float xp = __fadd_rn(1.0f, xi), den = fmaf(-2.0f * xi, u, xp);
+    const float mu = __fdividef(fmaf(-2.0f, u, xp), den);
+    const float om = __fdividef(2.0f * u * __fsub_rn(1.0f, xi), den);
+    const float sc = sqrtf(fmaxf(om * __fsub_rn(2.0f, om), 0.0f));
     const float v2 = fmaf(vx, vx, fmaf(vy, vy, vz * vz));
     float d0 = 0.0f, d1 = 0.0f, d2 = 1.0f;
     if (v2 > 0.0f) {
@@ -974,7 +974,7 @@ __device__ __forceinline__ float scatter32(float xi, float vx, float vy, float v
         d0 = vx * r; d1 = vy * r; d2 = vz * r;
     }
     const float sg = d2 >= 0.0f ? 1.0f : -1.0f;
-    const float a = -1.0f / (sg + d2);
+    const float a = -1.0f / __fadd_rn(sg, d2);
     const float b = d0 * d1 * a;
     float sn, cs;
     __sincosf(kTwoPiF * w, &sn, &cs);
@@ -1480,8 +1480,7 @@ struct Fp64Electron {
 // Each electron still takes exactly the sequence flight, collision,
 // flight, ... with the same random numbers.
 // Speed after an elastic collision that turns the direction from v to the
-// unit vector n (cos chi = mu when `given`, else from v and n), with the
-// recoil factor r: |v'| = |v| sqrt(1 - x), x = r (1 - cos chi), scaled on
+// unit vector n, with the recoil factor r: |v'| = |v| sqrt(1 - x), x = r (1 - cos chi), scaled on
 // the speed itself; a round trip through the energy would multiply by
 // (2a)_f32 * (1/2a)_f32 != 1 at every collision and drift.
 // |v| = v2 / sqrt(v2) from the hardware rsqrt with one Newton step in
@@ -1492,16 +1491,52 @@ struct Fp64Electron {
 // FMA: multiplying by a factor rounded just below 1.0 would bias it by
 // ~3e-10 per collision (a float32 emulation of both forms; this one is
 // unbiased).
-__device__ __forceinline__ float elastic_speed32(float vx, float vy, float vz, float nx, float ny,
-                                                 float nz, bool given, float mu, float recoil)
+//
+// Every rounding of the collision is written out (products fused or not as
+// stated): the warp's vote picks the straight-line or the general path, the
+// launch shape picks the build, and an electron's trajectory must not depend
+// on either.  A build's own choice of fused products did: two builds of the
+// general gas gave different electrons, and so did two runs of the basic gas
+// with crossings or signals, where the two paths differed.
+
+// |v|^2 of the isotropic collision and of the anisotropic one
+__device__ __forceinline__ float norm2_iso32(float x, float y, float z)
 {
-    const float v2 = vx * vx + vy * vy + vz * vz;
-    float r = rsqrtf(v2);
-    r = fmaf(r, fmaf(-0.5f * v2 * r, r, 0.5f), r);
-    const float cchi = given ? mu : (vx * nx + vy * ny + vz * nz) * r;
-    const float x = recoil * (1.0f - cchi);
-    const float vm = v2 * r, d = fmaf(0.125f * x, x, 0.5f * x);
+    return fmaf(z, z, fmaf(y, y, __fmul_rn(x, x)));
+}
+__device__ __forceinline__ float norm2_aniso32(float x, float y, float z)
+{
+    return __fadd_rn(fmaf(y, y, __fmul_rn(x, x)), __fmul_rn(z, z));
+}
+
+// |v'| from v2 = |v|^2, r ~ 1/|v| (speed_recip32) and om = 1 - cos chi.
+__device__ __forceinline__ float speed_recip32(float v2)
+{
+    const float r = rsqrtf(v2);
+    return fmaf(r, fmaf(__fmul_rn(__fmul_rn(-0.5f, v2), r), r, 0.5f), r);
+}
+__device__ __forceinline__ float recoil_speed32(float v2, float r, float om, float recoil)
+{
+    const float x = __fmul_rn(recoil, om);
+    const float vm = __fmul_rn(v2, r), d = fmaf(__fmul_rn(0.125f, x), x, __fmul_rn(0.5f, x));
     return v2 > 0.f ? fmaf(-vm, d, vm) : 0.f;
+}
+
+// isotropic: cos chi from v and n
+__device__ __forceinline__ float elastic_iso32(float vx, float vy, float vz, float nx, float ny,
+                                               float nz, float recoil)
+{
+    const float v2 = norm2_iso32(vx, vy, vz), r = speed_recip32(v2);
+    const float dn = fmaf(vz, nz, fmaf(vx, nx, __fmul_rn(vy, ny)));
+    return recoil_speed32(v2, r, fmaf(-dn, r, 1.0f), recoil);
+}
+
+// anisotropic: cos chi = mu as sampled
+__device__ __forceinline__ float elastic_aniso32(float vx, float vy, float vz, float mu,
+                                                 float recoil)
+{
+    const float v2 = norm2_aniso32(vx, vy, vz);
+    return recoil_speed32(v2, speed_recip32(v2), __fsub_rn(1.0f, mu), recoil);
 }
 
 struct MixedElectron {
@@ -1976,14 +2011,14 @@ struct MixedElectron {
         // the warp skips the search
         const bool lvl0 = (MAJ >= 1 || p.gas.level0_elastic) &&
                           __all_sync(__activemask(), pd.R < fmaf(pd.f, c0[tb.stride32] - c0[0], c0[0]));
-        if (lvl0 && !(PHYS && p.gas.any_aniso)) {
+        const bool aniso = PHYS && p.gas.any_aniso;
+        if (lvl0 && !aniso) {
             // the common case as straight-line code: every colliding lane of
             // the warp scatters elastically and isotropically on level 0
             ++n0;
             float nx, ny, nz;
             isotropic32(u01f(pd.w2), u01f(pd.w3), nx, ny, nz);
-            const float sp = elastic_speed32(vx, vy, vz, nx, ny, nz, false, 0.0f,
-                                             p.gas.recoil_f);
+            const float sp = elastic_iso32(vx, vy, vz, nx, ny, nz, p.gas.recoil_f);
             vx = sp * nx; vy = sp * ny; vz = sp * nz;
             ++nreal;
             if (p.coll_limit && nreal >= p.coll_limit) {
@@ -1993,7 +2028,8 @@ struct MixedElectron {
             return EV_NONE;
         }
         // the energy at the collision (the velocity has not changed since the flight)
-        const float eps = (vx * vx + vy * vy + vz * vz) * kInvTwoAccelF;
+        const float eps = __fmul_rn(aniso ? norm2_aniso32(vx, vy, vz) : norm2_iso32(vx, vy, vz),
+                                    kInvTwoAccelF);
         const int lvl = lvl0 ? 0 : select_below_total32(c0, tb.stride32, p.gas.n_levels, pd.f, pd.R);
         const int type = tb.type[lvl];
         if (type != GT_LEVEL_ELASTIC) {
@@ -2014,16 +2050,17 @@ struct MixedElectron {
         float sp;
         int ev = EV_NONE;
         float xi = 0.0f, mu = 0.0f;
-        if (PHYS && p.gas.any_aniso) {
+        if (aniso) {
             const float sc = tb.screen_f[lvl];
-            xi = sc > 0.0f ? __fdividef(eps, eps + sc) : tb.xi0_f[lvl];
+            xi = sc > 0.0f ? __fdividef(eps, __fadd_rn(eps, sc)) : tb.xi0_f[lvl];
         }
         if (xi != 0.0f)
             mu = scatter32(xi, vx, vy, vz, u01f(pd.w2), u01f(pd.w3), nx, ny, nz);
         else
             isotropic32(u01f(pd.w2), u01f(pd.w3), nx, ny, nz);
         if (type == GT_LEVEL_ELASTIC) {
-            sp = elastic_speed32(vx, vy, vz, nx, ny, nz, xi != 0.0f, mu, p.gas.recoil_f);
+            sp = xi != 0.0f ? elastic_aniso32(vx, vy, vz, mu, p.gas.recoil_f)
+                            : elastic_iso32(vx, vy, vz, nx, ny, nz, p.gas.recoil_f);
         } else {
             float eps_new = fmaxf(eps - tb.thr_f[lvl], 0.0f);
             if (type == GT_LEVEL_IONISATION) {

@@ -1,0 +1,35 @@
+"""Mixed precision, bit for bit: a run gives the same electrons again and with
+every launch shape, for both gases and every option that has builds of its own
+(the warp's vote and the build choose the code path, never the rounding)."""
+import numpy as np
+import pytest
+
+from paper_2509_15377_gb300 import avalanche as A
+from paper_2509_15377_gb300 import workloads as W
+from tests.gpu_helpers import by_uid, run_gpu
+
+pytestmark = pytest.mark.gpu
+
+SIGNAL = dict(signal_kind=W.W_PLATE, signal_bins=500, signal_dt=0.05)
+
+
+@pytest.mark.parametrize("gas", ["basic", "physical"])
+@pytest.mark.parametrize("option", [{}, {"crossing": 1}, SIGNAL, {"crossing": 1, **SIGNAL}])
+@pytest.mark.parametrize("majorant", [A.GT_MAJORANT_GLOBAL, A.GT_MAJORANT_BANDED])
+def test_same_electrons_again_and_with_every_shape(gas, option, majorant):
+    import __graft_entry__
+    __graft_entry__.build()
+    w = W.plate(n_avalanches=40, seed=9)
+    if gas == "physical":
+        w.gas = W.argon_like_physical_gas()
+    av = A.Avalanche(0)
+    av.set_gas(w.gas)
+    av.set_field(w.field)
+    runs = [by_uid(run_gpu(av, w, seed=9, precision=A.GT_MIXED, majorant=majorant,
+                           capacity=400_000, block=b, **option)[1])
+            for b in (0, 0, 512, 768, 896, 1024)]
+    av.close()
+    assert len(runs[0]["uid"]) > 1000
+    for r in runs[1:]:
+        for k in ("uid", "status", "n_flight", "x0", "e0", "x1", "y1", "z1", "t1", "e1", "tallies"):
+            assert np.array_equal(r[k], runs[0][k]), k
