@@ -161,7 +161,13 @@ Stack carve_stack(char *&p, int64_t cap)
     return s;
 }
 
-int default_block(int precision) { return precision == GT_FP64 ? 256 : 512; }
+// Warps per SM of an FP64 run: its FP64 pipe (2 lanes per clock) takes 16
+// clocks per warp instruction, so that five warps keep it busy and more only
+// lengthen each other's flights (300 avalanches of the 40 kV/cm plate:
+// 97 ms at 2 x 8 warps, 44.4 at 5; 46.9 at 4, 49.4 at 8, after the step itself became shorter).
+constexpr int kWarps64 = 5;
+
+int default_block(int precision) { return precision == GT_FP64 ? 32 * kWarps64 : 512; }
 
 // Which build of the mixed kernels a run uses (their launch shapes are tuned
 // apart): 0 the basic gas, 1 the general gas (anisotropy, attachment, a
@@ -353,7 +359,7 @@ static int gas_table_upload_impl(gt_ctx *ctx, const gt_gas *g)
     const int B = std::max(1, (N - 1 + bn - 1) / bn);
     int J = 0;
     while ((2 << J) <= B) ++J;
-    std::vector<double> band((size_t)(J + 1) * B);
+    std::vector<double> band((size_t)(J + 2) * B);  // and the first row's reciprocals
     for (int b = 0; b < B; ++b) {
         double m = 0.0;
         for (int k = b * bn; k <= (b + 1) * bn && k < N; ++k)
@@ -367,8 +373,9 @@ static int gas_table_upload_impl(gt_ctx *ctx, const gt_gas *g)
                                                        band[(size_t)(j - 1) * B + o])
                                             : band[(size_t)(j - 1) * B + b];
         }
-    std::vector<float> band32(band.size());
-    for (size_t i = 0; i < band.size(); ++i) band32[i] = (float)band[i];
+    for (int b = 0; b < B; ++b) band[(size_t)(J + 1) * B + b] = 1.0 / band[b];
+    std::vector<float> band32((size_t)(J + 1) * B);
+    for (size_t i = 0; i < band32.size(); ++i) band32[i] = (float)band[i];
 
     DeviceGuard dg(ctx->device);
     if (!dg.ok) return GT_ERR_CUDA;
@@ -421,6 +428,7 @@ static int gas_table_upload_impl(gt_ctx *ctx, const gt_gas *g)
     d.inv_band_width_f = (float)d.inv_band_width;
     d.last_band_f = (float)(B - 1);
     d.band64 = ctx->d_band64;
+    d.inv_band64 = ctx->d_band64 + (size_t)(J + 1) * B;
     d.band32 = ctx->d_band32;
     d.any_aniso = 0;
     for (int j = 0; j < L; ++j) {
@@ -1055,7 +1063,8 @@ static int plan_run(gt_ctx *ctx, const gt_run *r, const gt_endpoints *o, void *w
                 pl.smem = with;
             }
         }
-        pl.grid = r->grid ? r->grid : ctx->sms * occ;
+        const int per_sm = fp64 ? std::min(occ, std::max(1, 32 * kWarps64 / block)) : occ;
+        pl.grid = r->grid ? r->grid : ctx->sms * per_sm;
     }
     return GT_OK;
 }

@@ -49,6 +49,7 @@ struct DevGas {
     double inv_band_width;       // 1 / (n d_eps)
     float inv_band_width_f, last_band_f;
     const double *band64;        // [band_levels][n_bands]
+    const double *inv_band64;    // [n_bands] reciprocals of the first row
     const float *band32;
     int32_t type[GT_MAX_LEVELS];
     double thr[GT_MAX_LEVELS];
@@ -243,8 +244,12 @@ __device__ __forceinline__ uint4 draw_rk(const uint32_t (&rk)[20], int aval, uin
     return c;
 }
 
-// (w + 1/2) 2^-32 in (0, 1), exact in FP64.
-__device__ __forceinline__ double u01d(uint32_t w) { return ((double)w + 0.5) * 0x1p-32; }
+// (w + 1/2) 2^-32 in (0, 1), exact in FP64: 1 + w 2^-32 from its bits, less
+// 1 - 2^-33 (one FP64 instruction instead of a conversion and two).
+__device__ __forceinline__ double u01d(uint32_t w)
+{
+    return __hiloint2double((int)(0x3FF00000u | (w >> 12)), (int)(w << 20)) - (1.0 - 0x1p-33);
+}
 // (w>>9 + 1/2) 2^-23 in (0, 1), exact in FP32 (24 significant bits).  Built
 // from the bits (1 + (w>>9) 2^-23 has exponent 0) so that no int-to-float
 // conversion is issued: conversions share GB300's narrow FP64 pipe.
@@ -716,26 +721,35 @@ __device__ __forceinline__ void lorentz_step32(const DevField &f, float ax, floa
 }
 
 // Cumulative-rate selection at energy eps for R = u1 * nu_max: the level j
-// with cum_{j-1}(eps) <= R < cum_j(eps), or -1 for a null collision.
-template <typename R, typename T>
-__device__ __forceinline__ int select_level(const T *cum, int L, int N, R inv_d_eps, R eps, R Rv)
+// with cum_{j-1}(eps) <= R < cum_j(eps), or -1 for a null collision.  The
+// first level first (most real collisions are elastic), then a binary search
+// over the non-decreasing running sums: 3 to 15 FP64 instructions where a
+// count over all levels takes 33.
+__device__ __forceinline__ int select_level64(const double *cum, int L, int N, double inv_d_eps,
+                                              double eps, double Rv)
 {
-    R xk = eps * inv_d_eps;
-    const R last = (R)(N - 1);
-    if (xk > last) xk = last;
-    int k = (int)xk;
-    if (k > N - 2) k = N - 2;
-    const R f = xk - (R)k;
-    const T *c0 = cum + (int64_t)k * L;
-    const T *c1 = c0 + L;
-    const R top = (R)c0[L - 1] + f * ((R)c1[L - 1] - (R)c0[L - 1]);
-    if (!(Rv < top)) return -1;
-    int lvl = 0;
-    for (int j = 0; j < L - 1; ++j) {
-        const R cj = (R)c0[j] + f * ((R)c1[j] - (R)c0[j]);
-        lvl += (cj <= Rv) ? 1 : 0;
+    const double xk = fmin(eps * inv_d_eps, (double)(N - 1));
+    const int k = min((int)xk, N - 2);
+    const double f = xk - (double)k;
+    const double *c0 = cum + (int64_t)k * L;
+    const double *c1 = c0 + L;
+    const double a = __ldg(c0 + (L - 1)), b = __ldg(c1 + (L - 1));
+    const double a0 = __ldg(c0), b0 = __ldg(c1);
+    if (!(Rv < fma(f, b - a, a))) return -1;
+    if (Rv < fma(f, b0 - a0, a0)) return 0;
+    const int m = L - 1;  // the last level is known to exceed R
+    int pos = 1;          // the first is known not to
+    for (int n = m - 1; n > 0;) {
+        const int h = (n + 1) >> 1, j = pos + h - 1;
+        const double c = __ldg(c0 + j);
+        if (fma(f, __ldg(c1 + j) - c, c) <= Rv) {
+            pos += h;
+            n -= h;
+        } else {
+            n = h - 1;
+        }
     }
-    return lvl;
+    return pos;
 }
 
 // FP32 selection on a table with row stride `stride`, without int/float
@@ -787,11 +801,8 @@ __device__ __forceinline__ int select_below_total32(const float *c0, int stride,
 // Band of an energy: floor(eps / band width), clamped to the band range.
 __device__ __forceinline__ int band_index64(const DevGas &g, double eps)
 {
-    const double x = eps * g.inv_band_width;
-    if (!(x > 0.0)) return 0;
-    if (x >= (double)g.n_bands) return g.n_bands - 1;
-    const int b = (int)floor(x);
-    return b < g.n_bands ? b : g.n_bands - 1;
+    // the conversion truncates, saturates and takes a NaN to 0
+    return max(min(__double2int_rz(eps * g.inv_band_width), g.n_bands - 1), 0);
 }
 
 __device__ __forceinline__ int band_index32(const DevGas &g, float eps)
@@ -886,7 +897,7 @@ __device__ __forceinline__ void isotropic64(double u, double v, double &nx, doub
     const double st2 = 1.0 - ct * ct;
     const double st = st2 > 0.0 ? sqrt(st2) : 0.0;
     double s, c;
-    sincos(kTwoPi * v, &s, &c);
+    sincospi(2.0 * v, &s, &c);
     nx = st * c; ny = st * s; nz = ct;
 }
 
@@ -950,7 +961,7 @@ __device__ __forceinline__ double scatter64(double xi, double vx, double vy, dou
     const double a = -1.0 / (sg + d2);
     const double b = d0 * d1 * a;
     double sn, cs;
-    sincos(kTwoPi * w, &sn, &cs);
+    sincospi(2.0 * w, &sn, &cs);
     nx = mu * d0 + sc * (cs * (1.0 + sg * d0 * d0 * a) + sn * b);
     ny = mu * d1 + sc * (cs * (sg * b) + sn * (sg + d1 * d1 * a));
     nz = mu * d2 + sc * (cs * (-sg * d0) + sn * (-d1));
@@ -1248,15 +1259,23 @@ struct Fp64Electron {
         return status ? EV_RETIRE : EV_NONE;
     }
 
-    // Exact motion over dt with the acceleration a (and the field's B).
+    // Exact motion over dt with the acceleration a (and the field's B);
+    // z_only: the field is along z, so that without B x and y move uniformly.
     __device__ __forceinline__ void move(const RunParams &p, double ax, double ay, double az,
-                                         double dt)
+                                         double dt, bool z_only = false)
     {
         if (!p.field.has_b) {
-            x = x + vx * dt + 0.5 * ax * dt * dt;
-            y = y + vy * dt + 0.5 * ay * dt * dt;
-            z = z + vz * dt + 0.5 * az * dt * dt;
-            vx += ax * dt; vy += ay * dt; vz += az * dt;
+            const double h = 0.5 * dt;
+            if (z_only) {
+                x = fma(vx, dt, x);
+                y = fma(vy, dt, y);
+            } else {
+                x = fma(fma(h, ax, vx), dt, x);
+                y = fma(fma(h, ay, vy), dt, y);
+                vx = fma(ax, dt, vx); vy = fma(ay, dt, vy);
+            }
+            z = fma(fma(h, az, vz), dt, z);
+            vz = fma(az, dt, vz);
         } else {
             double dx, dy, dz;
             lorentz_step64(p.field, ax, ay, az, dt, vx, vy, vz, dx, dy, dz);
@@ -1345,14 +1364,26 @@ struct Fp64Electron {
         if (p.majorant == GT_MAJORANT_BANDED) {
             // the rate bound over the energies reachable within the window
             const double eps0 = (vx * vx + vy * vy + vz * vz) * kInvTwoAccel;
-            const double tau = p.window / __ldg(p.gas.band64 + band_index64(p.gas, eps0));
-            double lo, hi;
-            reach64(p.field.has_b, p.field_emax, eps0, vx, vy, vz, ex, ey, ez, tau, lo, hi);
-            nu = p.gas.bands_monotone
-                     ? __ldg(p.gas.band64 + band_index64(p.gas, hi))
-                     : band_range_max(p.gas.band64, p.gas.n_bands, band_index64(p.gas, lo),
-                                      band_index64(p.gas, hi));
-            dt = -log(u01d(w.x)) / nu;
+            const double tau = p.window * __ldg(p.gas.inv_band64 + band_index64(p.gas, eps0));
+            if (p.gas.bands_monotone && !p.field.has_b && p.field_emax <= 0.0) {
+                // bounds that rise with energy, a held field without B (the
+                // common run): the top band of the reach alone
+                const bool z_only = FK == GT_FIELD_PLATE || FK == GT_FIELD_UNIFORM;
+                const double vE = z_only ? vz * ez : vx * ex + vy * ey + vz * ez;
+                const double E2 = z_only ? ez * ez : ex * ex + ey * ey + ez * ez;
+                const double gw = (0.5 * kAccel * E2 * tau - vE) * tau;
+                const int top = band_index64(p.gas, eps0 + fmax(gw, 0.0));
+                nu = __ldg(p.gas.band64 + top);
+                dt = -log(u01d(w.x)) * __ldg(p.gas.inv_band64 + top);
+            } else {
+                double lo, hi;
+                reach64(p.field.has_b, p.field_emax, eps0, vx, vy, vz, ex, ey, ez, tau, lo, hi);
+                nu = p.gas.bands_monotone
+                         ? __ldg(p.gas.band64 + band_index64(p.gas, hi))
+                         : band_range_max(p.gas.band64, p.gas.n_bands, band_index64(p.gas, lo),
+                                          band_index64(p.gas, hi));
+                dt = -log(u01d(w.x)) / nu;
+            }
             if (dt >= tau) {
                 dt = tau;
                 pseudo = true;
@@ -1370,7 +1401,7 @@ struct Fp64Electron {
         if (p.substeps > 1 || p.crossing || p.signal_bins) {
             st = fly_steps<FK>(p, dt, ex, ey, ez, t_end);
         } else {
-            move(p, ax, ay, az, dt);
+            move(p, ax, ay, az, dt, FK == GT_FIELD_PLATE || FK == GT_FIELD_UNIFORM);
             st = boundary64<FK>(p.field, x, y, z);
         }
         t = t_end;
@@ -1384,9 +1415,10 @@ struct Fp64Electron {
             return EV_RETIRE;
         }
         if (pseudo) return EV_NONE;  // the window ended before a collision
-        const double eps = (vx * vx + vy * vy + vz * vz) * kInvTwoAccel;
-        int lvl = select_level<double, double>(tb.cum64, p.gas.n_levels, p.gas.n_nodes,
-                                                p.gas.inv_d_eps, eps, u01d(w.y) * nu);
+        const double v2 = vx * vx + vy * vy + vz * vz;
+        const double eps = v2 * kInvTwoAccel;
+        int lvl = select_level64(tb.cum64, p.gas.n_levels, p.gas.n_nodes, p.gas.inv_d_eps, eps,
+                                 u01d(w.y) * nu);
         if (lvl >= 0 && tb.type[lvl] != GT_LEVEL_ELASTIC && eps < tb.thr[lvl]) lvl = -1;
         if (lvl < 0) {
             ++nnull;
@@ -1407,8 +1439,7 @@ struct Fp64Electron {
         double eps_new;
         int ev = EV_NONE;
         if (type == GT_LEVEL_ELASTIC) {
-            const double sp = sqrt(vx * vx + vy * vy + vz * vz);
-            const double cchi = sp > 0.0 ? (vx * nx + vy * ny + vz * nz) / sp : 0.0;
+            const double cchi = v2 > 0.0 ? (vx * nx + vy * ny + vz * nz) * rsqrt(v2) : 0.0;
             eps_new = eps * (1.0 - p.gas.recoil * (1.0 - cchi));
         } else {
             eps_new = eps - tb.thr[lvl];
