@@ -90,8 +90,8 @@ static cudaError_t plain(const RunParams &p, const PlainArgs &a, int block, size
     const long long n = a.n_active;
     if (n <= 0) return cudaSuccess;
     k_plain_transport<MixedElectron, FK, TAB, kPlainThreadsMixed, PHYS, GEO>
-        <<<(unsigned)((n + block - 1) / block), block, smem, s>>>(p, a.cur, n, a.fresh, a.parity,
-                                                                  a.aval);
+        <<<plain_blocks(a, block), block, smem, s>>>(p, a.cur, n, a.lanes, a.fresh, a.parity,
+                                                     a.aval);
     return cudaGetLastError();
 }
 
