@@ -95,13 +95,14 @@ struct DevField {
 };
 
 struct Header {  // at the start of the work space, 256 bytes
-    unsigned long long head;      // next queue ticket
+    // (tail, done) and (head, error) are each read in one 16-byte access
     unsigned long long tail;      // slots reserved (stored or dropped)
     unsigned long long done;      // electrons finished or dropped
-    unsigned long long dropped;   // secondaries not stored
-    unsigned long long flights, real, nul;
+    unsigned long long head;      // next queue ticket
     unsigned int error;           // ERR_* bits
     unsigned int pad0;
+    unsigned long long dropped;   // secondaries not stored
+    unsigned long long flights, real, nul;
     unsigned long long n_new[2];  // plain mode: secondaries of this generation
     unsigned long long n_next[2]; // plain mode: electrons of next generation
     unsigned long long t_start;   // %globaltimer at the start of the run
@@ -131,7 +132,6 @@ struct RunParams {
     uint64_t *tallies;    // [n_avalanches][n_levels + 1]
     uint64_t *electrons;  // [n_avalanches]
     int64_t capacity;
-    int64_t n_primaries;  // slots below are primaries, the others new electrons
     // work space
     Header *hdr;
     unsigned int *ready;      // [capacity] queue slot filled
@@ -148,8 +148,6 @@ struct RunParams {
     int majorant;           // GT_MAJORANT_GLOBAL / GT_MAJORANT_BANDED
     double window;          // banded: window factor c
     float window_f;
-    int cell_off;           // MESH mixed: byte offset of the threads' elements in dynamic
-                            // shared memory (0: none)
     int substeps;           // field evaluations per flight (1: held field)
     int crossing;           // 1: leaving electrons end at the first crossing
     int signal_kind;        // readout electrode (GT_W_*), GT_W_NONE: no signal
@@ -163,6 +161,11 @@ struct RunParams {
     int n_avalanches;
     int aval_base;          // workload number of avalanche 0 (random-stream counter only)
     uint32_t rk[20];        // Philox round keys of the seed: (k0, k1) of rounds 0..9
+    // last, so that the fields above keep their places: shifted by 8 bytes they
+    // cost the plate's 1024-thread build 0.7 %
+    int64_t n_primaries;  // slots below are primaries, the others new electrons
+    int cell_off;           // MESH mixed: byte offset of the threads' elements in dynamic
+                            // shared memory (0: none)
 };
 
 // --------------------------------------------------------- small helpers
@@ -187,10 +190,21 @@ __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int *p)
     return v;
 }
 
-__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p)
+// Polls: no ordering, and the SM's L1 lines stay valid (an acquire drops them).
+__device__ __forceinline__ unsigned int ld_relaxed_u32(const unsigned int *p)
 {
-    unsigned long long v;
-    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    unsigned int v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Two neighbouring 64-bit words in one access of 16 bytes (16-byte aligned):
+// both as of the same moment.
+__device__ __forceinline__ ulonglong2 ld_relaxed_u64x2(const unsigned long long *p)
+{
+    ulonglong2 v;
+    asm volatile("{ .reg .b128 q; ld.relaxed.gpu.global.b128 q, [%2]; mov.b128 {%0, %1}, q; }"
+                 : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
     return v;
 }
 
@@ -1179,6 +1193,12 @@ __device__ __forceinline__ void signal_add(const RunParams &p, int aval, int nex
 }
 
 // ============================================================ FP64 electron
+// The FP64 pipe bounds this step: 2 lanes per clock, so 16 clocks per warp
+// instruction, and about 55 clocks from one result to the next.  Divisions by
+// tabulated rates go by tabulated reciprocals, the azimuth by sincospi, x and
+// y of a field along z move uniformly: 128 FP64 instructions per flight of the
+// plate instead of 201, a lone electron 10100 clocks per flight instead of
+// 15600 (300 avalanches at 40 kV/cm: 70 -> 47 ms at four warps per SM).
 struct Fp64Electron {
     static constexpr bool kTwoPhase = false;
     // New electron produced by an ionising collision (the parent supplies
@@ -1191,12 +1211,6 @@ struct Fp64Electron {
     double x, y, z, t, vx, vy, vz;
     double plate_e;
 
-// The FP64 pipe bounds this step: 2 lanes per clock, so 16 clocks per warp
-// instruction, and about 55 clocks from one result to the next.  Divisions by
-// tabulated rates go by tabulated reciprocals, the azimuth by sincospi, x and
-// y of a field along z move uniformly: 128 FP64 instructions per flight of the
-// plate instead of 201, a lone electron 10100 clocks per flight instead of
-// 15600 (300 avalanches at 40 kV/cm: 70 -> 47 ms at four warps per SM).
     __device__ __forceinline__ void bind(const Tables &) {}
     uint32_t nf, nreal, nnull;
     int status;

@@ -28,6 +28,8 @@ constexpr int kRoundCommon = 2;    // one flight per round, the step built for t
 constexpr int kRoundCrossing = 3;  // the same with exact crossings alone
 constexpr int kRoundSignal = 4;    // the same with induced signals alone
 
+constexpr int kFirstWarps = 4;     // of a CTA, see ticket_allowance
+
 // Row stride of the FP32 table staged in shared memory: odd, so that the
 // rows of a warp's random energies start on all 32 banks.
 __host__ __device__ inline int smem_stride(int n_levels) { return n_levels | 1; }
@@ -53,6 +55,7 @@ struct BlockState {
     unsigned long long flights, real, nul;
     unsigned long long last_done[32], last_tail[32], t_progress[32];
     unsigned int sleep_ns[32];
+    int allow[32];               // tickets the warp may take next (ticket_allowance)
     unsigned long long t_start;  // %globaltimer at the start of the run
 };
 
@@ -99,6 +102,7 @@ __device__ __forceinline__ Tables stage_tables(const RunParams &p, unsigned char
         bs.last_tail[threadIdx.x] = ~0ull;
         bs.t_progress[threadIdx.x] = 0ull;
         bs.sleep_ns[threadIdx.x] = 64u;
+        bs.allow[threadIdx.x] = 0;
     }
     __syncthreads();
     Tables tb;
@@ -198,6 +202,31 @@ __device__ __forceinline__ int push_children(const RunParams &p, bool want, cons
     return 0;
 }
 
+// Tickets a warp may take when the queue's counters read (head, tail);
+// `waits`: it has neither an electron nor a ticket.  While slots wait for
+// lanes, a warp takes its share of them (twice the even one, so that a full
+// queue fills every lane in a refill or two); while lanes wait for slots, one
+// lane of each SM's first warps holds a ticket.  The few electrons of a young
+// or a dying avalanche then run one or two per warp on every SM: in warps of 32
+// on the first SMs each lane waited for the others' branches (8 avalanches of
+// the 40 kV/cm plate: 1500-2000 cycles per round instead of 1170, 3.13 ms, now
+// 2.29; 2.71, 2.43, 2.29, 2.32 and 2.40 ms with 1, 2, 4, 8 and 32 first warps).
+// On a grid a warp takes tickets for all its idle lanes as it comes: the
+// slowest primary's drift sets the time there, and primaries that fill their
+// warps keep other avalanches' electrons, with rounds three times as long, out
+// of them (128 avalanches on a 256^3 grid: 109 ms, 114 with shares).
+template <int FK>
+__device__ __forceinline__ int ticket_allowance(unsigned long long head, unsigned long long tail,
+                                                bool waits)
+{
+    if (FK == GT_FIELD_GRID) return 32;
+    const int wid = threadIdx.x >> 5;
+    if (tail <= head) return waits && wid < kFirstWarps ? 1 : 0;
+    const unsigned a = (unsigned)min(tail - head, 1ull << 28);
+    if (wid >= kFirstWarps && a < gridDim.x) return 0;
+    return (int)(2u * a / ((blockDim.x >> 5) * gridDim.x) + 1u);
+}
+
 template <class E, int FK, bool SMEM_TABLE, int MAXT, int MP = 0, bool PHYS = true,
           bool GEO = true>
 __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
@@ -233,18 +262,24 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
             pre_m = 0u;
         }
         // lanes without an electron take queue tickets: one atomic per warp
-        const bool need = !has && ticket < 0;
-        const unsigned m = __ballot_sync(FULL, need);
+        __syncwarp();  // lane 0's bs.allow[wid]
+        const unsigned m = __ballot_sync(FULL, !has && ticket < 0);
         if (m) {
-            const int leader = __ffs(m) - 1;
-            unsigned long long base = 0;
-            if (lane == leader) base = atomicAdd(&p.hdr->head, (unsigned long long)__popc(m));
-            base = __shfl_sync(FULL, base, leader);
-            if (need) ticket = (long long)(base + __popc(m & lanemask_lt()));
+            const int take = min(bs.allow[wid], __popc(m));
+            if (take) {
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(&p.hdr->head, (unsigned long long)take);
+                base = __shfl_sync(FULL, base, 0);
+                const int rank = __popc(m & lanemask_lt());
+                if (((m >> lane) & 1u) && rank < take) ticket = (long long)(base + rank);
+            }
         }
         int retired = 0;
+        const bool busy = __any_sync(FULL, has);
         if (!has && ticket >= 0 && ticket < p.capacity) {
-            if (ld_acquire_u32(p.ready + ticket)) {
+            // an idle warp polls without ordering (the flag, once set, stays
+            // set); the acquiring read orders the record after the flag
+            if ((busy || ld_relaxed_u32(p.ready + ticket)) && ld_acquire_u32(p.ready + ticket)) {
                 e.template load_birth<FK, GEO>(p, ticket);
                 ticket = -1;
                 has = true;
@@ -267,11 +302,16 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
                 if (lane == 0) atomicAdd(&p.hdr->done, (unsigned long long)r);
                 continue;
             }
+            const bool waiting = __any_sync(FULL, ticket >= 0);
             int verdict = 0;  // 0 wait, 1 finished, 2 give up
             if (lane == 0) {
-                const unsigned long long d = ld_acquire_u64(&p.hdr->done);
-                const unsigned long long tl = ld_acquire_u64(&p.hdr->tail);
-                const unsigned err = *reinterpret_cast<volatile unsigned *>(&p.hdr->error);
+                // an electron's children are counted in tail before it is counted
+                // in done, so that equal counts of one moment mean the end
+                const ulonglong2 td = ld_relaxed_u64x2(&p.hdr->tail);
+                const ulonglong2 he = ld_relaxed_u64x2(&p.hdr->head);
+                const unsigned long long tl = td.x, d = td.y;
+                const unsigned err = (unsigned)he.y;
+                bs.allow[wid] = ticket_allowance<FK>(he.x, tl, !waiting);
                 const unsigned long long now = globaltimer();
                 if (d == tl) {
                     verdict = 1;
@@ -336,7 +376,10 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
             }
             // the lanes that will need an electron ask for tickets now
             if constexpr (kPrefetch) {
-                pre_m = __ballot_sync(FULL, !has && ticket < 0);
+                const unsigned idle = __ballot_sync(FULL, !has && ticket < 0);
+                // the first idle lanes, as many as the warp may take
+                pre_m = __ballot_sync(FULL, ((idle >> lane) & 1u) &&
+                                                __popc(idle & lanemask_lt()) < bs.allow[wid]);
                 if (pre_m && lane == __ffs(pre_m) - 1)
                     pre_base = atomicAdd(&p.hdr->head, (unsigned long long)__popc(pre_m));
             }
@@ -370,7 +413,10 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
         // the run-wide checks: the time budget, and an abort from any warp
         unsigned stop = 0;
         if (lane == 0) {
-            const unsigned err = *reinterpret_cast<volatile unsigned *>(&p.hdr->error);
+            const ulonglong2 td = ld_relaxed_u64x2(&p.hdr->tail);
+            const ulonglong2 he = ld_relaxed_u64x2(&p.hdr->head);
+            const unsigned err = (unsigned)he.y;
+            bs.allow[wid] = ticket_allowance<FK>(he.x, td.x, false);
             if ((long long)(globaltimer() - bs.t_start) > p.time_limit_ns) {
                 atomicOr(&p.hdr->error, ERR_TIMEOUT);
                 stop = 1u;
