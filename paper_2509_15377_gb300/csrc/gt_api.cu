@@ -167,7 +167,27 @@ Stack carve_stack(char *&p, int64_t cap)
 // 97 ms at 2 x 8 warps, 44.4 at 5; 46.9 at 4, 49.4 at 8, after the step itself became shorter).
 constexpr int kWarps64 = 5;
 
-int default_block(int precision) { return precision == GT_FP64 ? 32 * kWarps64 : 512; }
+// Threads per CTA of a batched run that leaves them open.  Mixed: 512 (16 warps,
+// all the registers they want) has the shorter rounds, 1024 (64 registers, no
+// spills in the builds for the common run) the more electrons, and on a plate
+// it wins where the run is much longer than its longest chain: room for 32
+// electrons per lane of a full GPU and many primaries.  767 avalanches with
+// three primaries and the general gas: 21.5 ms at 512, 18.1 at 768, 16.8 at 1024;
+// 1000 avalanches (room for 11 per lane): 7.16, 7.06 and 7.18-7.38; with exact
+// crossings 8.07, 7.72 and 7.55; signals, whose state spills at 1024, 17.6, 16.9
+// and 17.9 ms.  The global majorant's long chains and the other fields' drifts
+// stay at 512 (500 avalanches: 17.0, 18.2, 22.1; the 256^3 grid 112, 132, 154).
+int default_block(const gt_ctx *ctx, const gt_run *r, int64_t capacity)
+{
+    if (r->precision == GT_FP64) return 32 * kWarps64;
+    const int64_t lanes = (int64_t)1024 * ctx->sms;
+    if (r->mode != GT_BATCHED || r->majorant != GT_MAJORANT_BANDED ||
+        ctx->field.kind != GT_FIELD_PLATE || ctx->field.has_b || r->substeps > 1 ||
+        r->n_primaries < 2 * ctx->sms || capacity < 8 * lanes)
+        return 512;
+    const bool signal = r->signal_kind != GT_W_NONE && r->signal_bins > 0;
+    return capacity >= 32 * lanes && !signal ? 1024 : 768;
+}
 
 // Which build of the mixed kernels a run uses (their launch shapes are tuned
 // apart): 0 the basic gas, 1 the general gas (anisotropy, attachment, a
@@ -1037,7 +1057,7 @@ static int plan_run(gt_ctx *ctx, const gt_run *r, const gt_endpoints *o, void *w
     const int tuned_b = ctx->tuned_block[prec_i][ctx->field.kind][maj_i][var_i];
     const int block = r->block ? r->block
                                : (r->mode == GT_BATCHED && tuned_b > 0 ? tuned_b
-                                                                       : default_block(r->precision));
+                                                                       : default_block(ctx, r, o->capacity));
     const int band_entries = ctx->gas.n_bands * ctx->gas.band_levels;
     const size_t smem_tab = shared_bytes(L, ctx->gas.n_nodes, block, true, band_entries);
     const size_t smem_cap = ctx->smem_optin - kStaticSmemReserve;
