@@ -44,6 +44,16 @@ static bool signal_only_run(const RunParams &p)
     return common_run(p) && p.signal_bins > 0 && !p.crossing && p.substeps <= 1;
 }
 
+// The global majorant without B (kRoundGlobal, the plate and uniform fields in
+// the basic variant).
+template <int FK, bool PHYS, bool GEO>
+constexpr bool kHasGlobal = !PHYS && !GEO && (FK == GT_FIELD_PLATE || FK == GT_FIELD_UNIFORM);
+
+static bool global_run(const RunParams &p)
+{
+    return p.majorant == GT_MAJORANT_GLOBAL && !p.field.has_b && p.flights_per_phase > 1;
+}
+
 template <int FK, bool TAB, int MAXT, bool PHYS, bool GEO>
 static cudaError_t batched_t(const RunParams &p, int grid, int block, size_t smem, cudaStream_t s)
 {
@@ -63,6 +73,13 @@ static cudaError_t batched_t(const RunParams &p, int grid, int block, size_t sme
     if constexpr ((!PHYS && !GEO) || FK == GT_FIELD_PLATE) {
         if (common_run(p)) {
             k_batched<MixedElectron, FK, TAB, MAXT, kRoundCommon, PHYS, GEO>
+                <<<grid, block, smem, s>>>(p);
+            return cudaGetLastError();
+        }
+    }
+    if constexpr (kHasGlobal<FK, PHYS, GEO>) {
+        if (global_run(p)) {
+            k_batched<MixedElectron, FK, TAB, MAXT, kRoundGlobal, PHYS, GEO>
                 <<<grid, block, smem, s>>>(p);
             return cudaGetLastError();
         }
@@ -177,6 +194,9 @@ static cudaError_t configure_one(size_t max_smem)
     if ((e = configure_mp<FK, TAB, kRoundOne, PHYS, GEO>(max_smem)) != cudaSuccess) return e;
     if constexpr ((!PHYS && !GEO) || FK == GT_FIELD_PLATE) {
         if ((e = configure_mp<FK, TAB, kRoundCommon, PHYS, GEO>(max_smem)) != cudaSuccess) return e;
+    }
+    if constexpr (kHasGlobal<FK, PHYS, GEO>) {
+        if ((e = configure_mp<FK, TAB, kRoundGlobal, PHYS, GEO>(max_smem)) != cudaSuccess) return e;
     }
     if constexpr (GEO && FK == GT_FIELD_PLATE) {
         if ((e = configure_mp<FK, TAB, kRoundCrossing, PHYS, GEO>(max_smem)) != cudaSuccess) return e;

@@ -33,3 +33,25 @@ def test_same_electrons_again_and_with_every_shape(gas, option, majorant):
     for r in runs[1:]:
         for k in ("uid", "status", "n_flight", "x0", "e0", "x1", "y1", "z1", "t1", "e1", "tallies"):
             assert np.array_equal(r[k], runs[0][k]), k
+
+
+@pytest.mark.parametrize("gas", ["drift", "argon"])
+@pytest.mark.parametrize("phase", [2, 6])
+def test_global_majorant_build_equals_the_general_one(gas, phase):
+    """In the unbounded uniform field the option of exact crossings changes
+    nothing but the build: the global majorant's own and the general one give
+    the same electrons bit for bit."""
+    import __graft_entry__
+    __graft_entry__.build()
+    w = W.drift_model(n_electrons=100, n_coll=500, e_field=20_000.0, seed=12)
+    if gas == "argon":
+        w.gas = W.argon_like_gas()
+    av = A.Avalanche(0)
+    av.set_gas(w.gas)
+    av.set_field(w.field)
+    a, b = (by_uid(run_gpu(av, w, seed=12, precision=A.GT_MIXED, majorant=A.GT_MAJORANT_GLOBAL,
+                           flights_per_phase=phase, capacity=400_000, crossing=c)[1])
+            for c in (0, 1))
+    av.close()
+    for k in ("uid", "status", "n_flight", "x0", "x1", "y1", "z1", "t1", "e1", "tallies"):
+        assert np.array_equal(a[k], b[k]), k
