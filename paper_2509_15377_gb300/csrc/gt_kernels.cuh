@@ -213,15 +213,9 @@ __device__ __forceinline__ int push_children(const RunParams &p, bool want, cons
 // on the first SMs each lane waited for the others' branches (8 avalanches of
 // the 40 kV/cm plate: 1500-2000 cycles per round instead of 1170, 3.13 ms, now
 // 2.29; 2.71, 2.43, 2.29, 2.32 and 2.40 ms with 1, 2, 4, 8 and 32 first warps).
-// On a grid a warp takes tickets for all its idle lanes as it comes: the
-// slowest primary's drift sets the time there, and primaries that fill their
-// warps keep other avalanches' electrons, with rounds three times as long, out
-// of them (128 avalanches on a 256^3 grid: 109 ms, 114 with shares).
-template <int FK>
 __device__ __forceinline__ int ticket_allowance(unsigned long long head, unsigned long long tail,
                                                 bool waits)
 {
-    if (FK == GT_FIELD_GRID) return 32;
     const int wid = threadIdx.x >> 5;
     if (tail <= head) return waits && wid < kFirstWarps ? 1 : 0;
     const unsigned a = (unsigned)min(tail - head, 1ull << 28);
@@ -254,6 +248,14 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
     // the common-run builds without sub-steps, crossings or signals, whose
     // registers have room for it
     constexpr bool kPrefetch = MP == kRoundCommon && !GEO;
+    // shares of the queue (ticket_allowance) in the builds for up to 768 threads;
+    // the others take tickets for all their idle lanes as they come: their runs
+    // are full nearly from start to end, and reading tail between its atomics
+    // costs a full GPU 3 % (4096 avalanches 90.1 -> 87.4 ms without it).  The same
+    // on a grid: the slowest primary's drift sets the time there, and primaries
+    // that fill their warps keep other avalanches' electrons, with rounds three
+    // times as long, out of them (128 avalanches on a 256^3 grid: 114 -> 105 ms).
+    constexpr bool kShares = FK != GT_FIELD_GRID && MAXT <= 768;
     unsigned pre_m = 0u;
     unsigned long long pre_base = 0ull;
     for (; !stop0;) {
@@ -267,7 +269,7 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
         __syncwarp();  // lane 0's bs.allow[wid]
         const unsigned m = __ballot_sync(FULL, !has && ticket < 0);
         if (m) {
-            const int take = min(bs.allow[wid], __popc(m));
+            const int take = kShares ? min(bs.allow[wid], __popc(m)) : __popc(m);
             if (take) {
                 unsigned long long base = 0;
                 if (lane == 0) base = atomicAdd(&p.hdr->head, (unsigned long long)take);
@@ -304,16 +306,16 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
                 if (lane == 0) atomicAdd(&p.hdr->done, (unsigned long long)r);
                 continue;
             }
-            const bool waiting = __any_sync(FULL, ticket >= 0);
+            const bool waiting = !kShares || __any_sync(FULL, ticket >= 0);
             int verdict = 0;  // 0 wait, 1 finished, 2 give up
             if (lane == 0) {
                 // an electron's children are counted in tail before it is counted
                 // in done, so that equal counts of one moment mean the end
                 const ulonglong2 td = ld_relaxed_u64x2(&p.hdr->tail);
-                const ulonglong2 he = ld_relaxed_u64x2(&p.hdr->head);
+                const unsigned err = ld_relaxed_u32(&p.hdr->error);
                 const unsigned long long tl = td.x, d = td.y;
-                const unsigned err = (unsigned)he.y;
-                bs.allow[wid] = ticket_allowance<FK>(he.x, tl, !waiting);
+                if (kShares)
+                    bs.allow[wid] = ticket_allowance(ld_relaxed_u64(&p.hdr->head), tl, !waiting);
                 const unsigned long long now = globaltimer();
                 if (d == tl) {
                     verdict = 1;
@@ -383,7 +385,7 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
                 const unsigned idle = __ballot_sync(FULL, !has && ticket < 0);
                 // the first idle lanes, as many as the warp may take
                 pre_m = __ballot_sync(FULL, ((idle >> lane) & 1u) &&
-                                                __popc(idle & lanemask_lt()) < bs.allow[wid]);
+                                                (!kShares || __popc(idle & lanemask_lt()) < bs.allow[wid]));
                 if (pre_m && lane == __ffs(pre_m) - 1)
                     pre_base = atomicAdd(&p.hdr->head, (unsigned long long)__popc(pre_m));
             }
@@ -417,10 +419,11 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
         // the run-wide checks: the time budget, and an abort from any warp
         unsigned stop = 0;
         if (lane == 0) {
-            const ulonglong2 td = ld_relaxed_u64x2(&p.hdr->tail);
-            const ulonglong2 he = ld_relaxed_u64x2(&p.hdr->head);
-            const unsigned err = (unsigned)he.y;
-            bs.allow[wid] = ticket_allowance<FK>(he.x, td.x, false);
+            const unsigned err = ld_relaxed_u32(&p.hdr->error);
+            if constexpr (kShares) {
+                const unsigned long long tl = ld_relaxed_u64(&p.hdr->tail);
+                bs.allow[wid] = ticket_allowance(ld_relaxed_u64(&p.hdr->head), tl, false);
+            }
             if ((long long)(globaltimer() - bs.t_start) > p.time_limit_ns) {
                 atomicOr(&p.hdr->error, ERR_TIMEOUT);
                 stop = 1u;
