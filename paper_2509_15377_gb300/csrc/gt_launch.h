@@ -18,14 +18,11 @@ int context_device(const gt_ctx *ctx);
 constexpr size_t kStaticSmemReserve = 4096;
 
 // Let a kernel use all the dynamic shared memory a CTA may have beyond the
-// kernel's own static shared memory.
+// reserve (one call per kernel: gt_create makes 500 of them).
 template <typename F>
 inline cudaError_t allow_dynamic_smem(F *kernel, size_t optin)
 {
-    cudaFuncAttributes a;
-    cudaError_t e = cudaFuncGetAttributes(&a, kernel);
-    if (e != cudaSuccess) return e;
-    const size_t dyn = optin > a.sharedSizeBytes ? optin - a.sharedSizeBytes : 0;
+    const size_t dyn = optin > kStaticSmemReserve ? optin - kStaticSmemReserve : 0;
     return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
 }
 
