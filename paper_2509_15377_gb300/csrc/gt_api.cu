@@ -170,13 +170,15 @@ constexpr int kWarps64 = 5;
 // Threads per CTA of a batched run that leaves them open.  Mixed: 512 (16 warps,
 // all the registers they want) has the shorter rounds, 1024 (64 registers, no
 // spills in the builds for the common run) the more electrons, and on a plate
-// it wins where the run is much longer than its longest chain: room for 32
-// electrons per lane of a full GPU and many primaries.  767 avalanches with
-// three primaries and the general gas: 21.5 ms at 512, 18.1 at 768, 16.8 at 1024;
-// 1000 avalanches (room for 11 per lane): 7.16, 7.06 and 7.18-7.38; with exact
-// crossings 8.07, 7.72 and 7.55; signals, whose state spills at 1024, 17.6, 16.9
-// and 17.9 ms.  The global majorant's long chains and the other fields' drifts
-// stay at 512 (500 avalanches: 17.0, 18.2, 22.1; the 256^3 grid 112, 132, 154).
+// it wins where the run is much longer than its longest chain: many primaries
+// and room for many electrons per lane of a full GPU.  At 512, 768, 896 and 1024:
+// 1000 avalanches of the 40 kV/cm plate (room for 11 per lane) 7.18, 7.15, 6.68
+// and 6.73 ms; 767 avalanches with three primaries and the general gas (50 per
+// lane) 21.6, 18.4, 16.6 and 16.1; exact crossings (11 per lane) 7.87, 7.18, 7.36
+// and 7.31; signals, whose state spills beyond 768, 18.5, 16.6, 16.7 and 17.8; 8
+// avalanches 2.27, 2.63, 3.7 and 3.7.  The global majorant's long chains and the
+// other fields' drifts stay at 512 (500 avalanches 17.0 at 512, 22.1 at 1024; the
+// 256^3 grid 112 and 154).
 int default_block(const gt_ctx *ctx, const gt_run *r, int64_t capacity)
 {
     if (r->precision == GT_FP64) return 32 * kWarps64;
@@ -185,8 +187,9 @@ int default_block(const gt_ctx *ctx, const gt_run *r, int64_t capacity)
         ctx->field.kind != GT_FIELD_PLATE || ctx->field.has_b || r->substeps > 1 ||
         r->n_primaries < 2 * ctx->sms || capacity < 8 * lanes)
         return 512;
-    const bool signal = r->signal_kind != GT_W_NONE && r->signal_bins > 0;
-    return capacity >= 32 * lanes && !signal ? 1024 : 768;
+    if (r->signal_kind != GT_W_NONE && r->signal_bins > 0) return 768;
+    if (capacity >= 32 * lanes) return 1024;
+    return r->crossing ? 768 : 896;
 }
 
 // Which build of the mixed kernels a run uses (their launch shapes are tuned
@@ -1041,18 +1044,6 @@ static int plan_run(gt_ctx *ctx, const gt_run *r, const gt_endpoints *o, void *w
         sa.dx = r->dx; sa.dy = r->dy; sa.dz = r->dz; sa.aval = r->aval; sa.uid = r->uid;
     }
 
-    // outputs and queue flags start from zero
-    if (o->capacity > 0)
-        GT_CUDA(ctx, cudaMemsetAsync(p.ready, 0, sizeof(uint32_t) * (size_t)o->capacity, s));
-    if (na > 0) {
-        GT_CUDA(ctx, cudaMemsetAsync(o->tallies, 0, sizeof(uint64_t) * (size_t)na * (L + 1), s));
-        if (p.signal_bins)
-            GT_CUDA(ctx, cudaMemsetAsync(o->signal, 0,
-                                         sizeof(double) * (size_t)na * (size_t)p.signal_bins, s));
-        GT_CUDA(ctx, cudaMemsetAsync(o->electrons, 0, sizeof(uint64_t) * (size_t)na, s));
-        if (r->size_limit)
-            GT_CUDA(ctx, cudaMemsetAsync(p.created, 0, sizeof(unsigned long long) * (size_t)na, s));
-    }
     const bool fp64 = r->precision == GT_FP64;
     const int tuned_b = ctx->tuned_block[prec_i][ctx->field.kind][maj_i][var_i];
     const int block = r->block ? r->block
