@@ -27,6 +27,7 @@ constexpr int kRoundOne = 1;       // one flight per round
 constexpr int kRoundCommon = 2;    // one flight per round, the step built for the common run
 constexpr int kRoundCrossing = 3;  // the same with exact crossings alone
 constexpr int kRoundSignal = 4;    // the same with induced signals alone
+constexpr int kRoundCommonB = 6;   // the common run's round and step in a magnetic field
 constexpr int kRoundGlobal = 5;    // flights per round from the run, the step built for the
                                    // global majorant without B
 
@@ -350,9 +351,10 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
             // MAJ = 1), and with exact crossings / induced signals alone
             // (MAJ = 2 / 3)
             constexpr int MPF = MP == kRoundGlobal ? 0 : MP >= kRoundCommon ? 1 : MP;
-            constexpr int MAJ = MP == kRoundGlobal   ? kMajGlobal
-                                : MP >= kRoundCommon ? MP - kRoundOne
-                                                     : 0;
+            constexpr int MAJ = MP == kRoundGlobal    ? kMajGlobal
+                                : MP == kRoundCommonB ? kMajBandedB
+                                : MP >= kRoundCommon  ? MP - kRoundOne
+                                                      : 0;
             const int M = MPF ? MPF : p.flights_per_phase;
             // an electron that finishes during the rounds keeps its lane (a
             // lane takes a new electron only at the next refill) and is

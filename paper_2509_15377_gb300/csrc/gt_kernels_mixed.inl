@@ -23,12 +23,18 @@ constexpr int kPlainThreadsMixed = 512;
 // The run the step has a build of its own for (kRoundCommon): one flight per
 // round, the banded majorant with band bounds rising with energy, an
 // elastic level 0, no magnetic field, the field held over each flight.
-static bool common_run(const RunParams &p)
+static bool common_but_b(const RunParams &p)
 {
     return p.flights_per_phase == 1 && p.majorant == GT_MAJORANT_BANDED &&
-           p.gas.bands_monotone && p.gas.level0_elastic && !p.field.has_b &&
-           p.field_emax_f == 0.0f;
+           p.gas.bands_monotone && p.gas.level0_elastic && p.field_emax_f == 0.0f;
 }
+
+static bool common_run(const RunParams &p) { return common_but_b(p) && !p.field.has_b; }
+
+// The common run in a magnetic field (kRoundCommonB, the tube in the basic
+// variant).
+template <int FK, bool PHYS, bool GEO>
+constexpr bool kHasCommonB = !PHYS && !GEO && FK == GT_FIELD_COAX;
 
 // The common run with exact crossings and neither sub-steps nor signals
 // (kRoundCrossing, the plate field in the GEO variant).
@@ -73,6 +79,13 @@ static cudaError_t batched_t(const RunParams &p, int grid, int block, size_t sme
     if constexpr ((!PHYS && !GEO) || FK == GT_FIELD_PLATE) {
         if (common_run(p)) {
             k_batched<MixedElectron, FK, TAB, MAXT, kRoundCommon, PHYS, GEO>
+                <<<grid, block, smem, s>>>(p);
+            return cudaGetLastError();
+        }
+    }
+    if constexpr (kHasCommonB<FK, PHYS, GEO>) {
+        if (common_but_b(p) && p.field.has_b) {
+            k_batched<MixedElectron, FK, TAB, MAXT, kRoundCommonB, PHYS, GEO>
                 <<<grid, block, smem, s>>>(p);
             return cudaGetLastError();
         }
@@ -194,6 +207,9 @@ static cudaError_t configure_one(size_t max_smem)
     if ((e = configure_mp<FK, TAB, kRoundOne, PHYS, GEO>(max_smem)) != cudaSuccess) return e;
     if constexpr ((!PHYS && !GEO) || FK == GT_FIELD_PLATE) {
         if ((e = configure_mp<FK, TAB, kRoundCommon, PHYS, GEO>(max_smem)) != cudaSuccess) return e;
+    }
+    if constexpr (kHasCommonB<FK, PHYS, GEO>) {
+        if ((e = configure_mp<FK, TAB, kRoundCommonB, PHYS, GEO>(max_smem)) != cudaSuccess) return e;
     }
     if constexpr (kHasGlobal<FK, PHYS, GEO>) {
         if ((e = configure_mp<FK, TAB, kRoundGlobal, PHYS, GEO>(max_smem)) != cudaSuccess) return e;

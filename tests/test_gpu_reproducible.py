@@ -55,3 +55,28 @@ def test_global_majorant_build_equals_the_general_one(gas, phase):
     av.close()
     for k in ("uid", "status", "n_flight", "x0", "x1", "y1", "z1", "t1", "e1", "tallies"):
         assert np.array_equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("tilt", [(0.0, 0.0, 1.0), (0.0, 0.0, -2.5)])
+def test_tube_build_with_b_equals_the_general_one(tilt):
+    """The tube's own build for B needs band bounds that rise with energy; a gas
+    whose last band (99-100 eV, beyond every electron here) falls takes the
+    build for any run, with the same bounds below."""
+    import __graft_entry__
+    __graft_entry__.build()
+    w = W.coax(n_avalanches=64, r_lo=0.01, r_hi=0.03, seed=13)
+    w.field.b = tilt
+    av = A.Avalanche(0)
+    runs = []
+    for falling in (False, True):
+        g = W.argon_like_gas()
+        if falling:
+            g.rate[1980:, 0] = 0.0
+        av.set_gas(g)
+        av.set_field(w.field)
+        runs.append(by_uid(run_gpu(av, w, seed=13, precision=A.GT_MIXED, majorant=1,
+                                   t_max=0.5, capacity=400_000)[1]))
+    av.close()
+    assert len(runs[0]["uid"]) >= 64 and max(r["e1"].max() for r in runs) < 95.0
+    for k in ("uid", "status", "n_flight", "x0", "x1", "y1", "z1", "t1", "e1", "tallies"):
+        assert np.array_equal(runs[0][k], runs[1][k]), k
