@@ -1046,12 +1046,17 @@ static int plan_run(gt_ctx *ctx, const gt_run *r, const gt_endpoints *o, void *w
 
     const bool fp64 = r->precision == GT_FP64;
     const int tuned_b = ctx->tuned_block[prec_i][ctx->field.kind][maj_i][var_i];
-    const int block = r->block ? r->block
-                               : (r->mode == GT_BATCHED && tuned_b > 0 ? tuned_b
-                                                                       : default_block(ctx, r, o->capacity));
     const int band_entries = ctx->gas.n_bands * ctx->gas.band_levels;
-    const size_t smem_tab = shared_bytes(L, ctx->gas.n_nodes, block, true, band_entries);
     const size_t smem_cap = ctx->smem_optin - kStaticSmemReserve;
+    int block = r->block ? r->block : r->mode == GT_BATCHED ? tuned_b : 0;
+    if (!block) {
+        // more threads only while the gas table still fits beside their state
+        block = default_block(ctx, r, o->capacity);
+        while (!fp64 && block > 512 &&
+               shared_bytes(L, ctx->gas.n_nodes, block, true, band_entries) > smem_cap)
+            block = block > 896 ? 896 : block > 768 ? 768 : 512;
+    }
+    const size_t smem_tab = shared_bytes(L, ctx->gas.n_nodes, block, true, band_entries);
     const bool smem_table = !fp64 && smem_tab <= smem_cap;
     const size_t smem = shared_bytes(L, ctx->gas.n_nodes, block, smem_table, band_entries);
     if (smem > smem_cap) return GT_ERR_UNSUPPORTED;
