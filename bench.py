@@ -53,13 +53,14 @@ WORKLOAD = "plate_batched_4096"
 #   level choice, tally, isotropic direction and speed), counted from its
 #   arithmetic, one lane instruction per operation; what the kernel issues
 #   beyond it (spill code, addressing, control, FP64 folds) is overhead.
-LANE_INST_PER_FLIGHT_BY_BLOCK = {768: 321.2, 896: 323.2, 1024: 313.5}
+LANE_INST_PER_FLIGHT_BY_BLOCK = {768: 332.8, 896: 310.0, 1024: 302.1}
 ALGORITHMIC_LANE_INST_PER_FLIGHT = 190.0
 # The same calibration for the field-map line on the 256^3 grid (`bench.py
-# --calibrate --calibrate-field grid --block B --refill-period 16
+# --calibrate --calibrate-field grid --block B --refill-period 32 (16 for 768
+# and 1024 threads)
 # --flights-per-phase 1`: straight-line flights at r = 1 mm in the map, the
 # step plus eight float4 gathers and the trilinear interpolation per flight).
-GRID_LANE_INST_PER_FLIGHT_BY_BLOCK = {512: 419.7, 768: 442.3, 1024: 414.1}
+GRID_LANE_INST_PER_FLIGHT_BY_BLOCK = {512: 403.9, 768: 442.3, 1024: 414.1}
 
 
 def lane_inst_per_flight(block: int, table=None) -> float:
