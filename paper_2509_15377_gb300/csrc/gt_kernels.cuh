@@ -207,9 +207,11 @@ __device__ __forceinline__ int push_children(const RunParams &p, bool want, cons
 
 // Tickets a warp may take when the queue's counters read (head, tail);
 // `waits`: it has neither an electron nor a ticket.  While slots wait for
-// lanes, a warp takes its share of them (twice the even one, so that a full
-// queue fills every lane in a refill or two); while lanes wait for slots, one
-// lane of each SM's first warps holds a ticket.  The few electrons of a young
+// lanes, a warp takes them for all its idle lanes when there is one and more
+// for every warp (smaller shares left lanes idle for several refills: 116,736
+// electrons that start at once at 768 threads 2.52 ms, now 1.78), else twice
+// the even share; while lanes wait for slots, one lane of each SM's first warps
+// holds a ticket.  The few electrons of a young
 // or a dying avalanche then run one or two per warp on every SM: in warps of 32
 // on the first SMs each lane waited for the others' branches (8 avalanches of
 // the 40 kV/cm plate: 1500-2000 cycles per round instead of 1170, 3.13 ms, now
@@ -221,7 +223,8 @@ __device__ __forceinline__ int ticket_allowance(unsigned long long head, unsigne
     if (tail <= head) return waits && wid < kFirstWarps ? 1 : 0;
     const unsigned a = (unsigned)min(tail - head, 1ull << 28);
     if (wid >= kFirstWarps && a < gridDim.x) return 0;
-    return (int)(2u * a / ((blockDim.x >> 5) * gridDim.x) + 1u);
+    const unsigned warps = (blockDim.x >> 5) * gridDim.x;
+    return a >= warps ? 32 : (int)(2u * a / warps + 1u);
 }
 
 template <class E, int FK, bool SMEM_TABLE, int MAXT, int MP = 0, bool PHYS = true,
