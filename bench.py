@@ -53,7 +53,7 @@ WORKLOAD = "plate_batched_4096"
 #   level choice, tally, isotropic direction and speed), counted from its
 #   arithmetic, one lane instruction per operation; what the kernel issues
 #   beyond it (spill code, addressing, control, FP64 folds) is overhead.
-LANE_INST_PER_FLIGHT_BY_BLOCK = {768: 332.8, 896: 310.0, 1024: 302.1}
+LANE_INST_PER_FLIGHT_BY_BLOCK = {768: 322.6, 896: 310.0, 1024: 302.1}
 ALGORITHMIC_LANE_INST_PER_FLIGHT = 190.0
 # The same calibration for the field-map line on the 256^3 grid (`bench.py
 # --calibrate --calibrate-field grid --block B --refill-period 32 (16 for 768
