@@ -211,11 +211,11 @@ __device__ __forceinline__ int push_children(const RunParams &p, bool want, cons
 // for every warp (smaller shares left lanes idle for several refills: 116,736
 // electrons that start at once at 768 threads 2.52 ms, now 1.78), else twice
 // the even share; while lanes wait for slots, one lane of each SM's first warps
-// holds a ticket.  The few electrons of a young
-// or a dying avalanche then run one or two per warp on every SM: in warps of 32
-// on the first SMs each lane waited for the others' branches (8 avalanches of
-// the 40 kV/cm plate: 1500-2000 cycles per round instead of 1170, 3.13 ms, now
-// 2.29; 2.71, 2.43, 2.29, 2.32 and 2.40 ms with 1, 2, 4, 8 and 32 first warps).
+// holds a ticket.  The few electrons of a young or a dying avalanche then run
+// one or two per warp on every SM: in warps of 32 on the first SMs each lane
+// waited for the others' branches (8 avalanches of the 40 kV/cm plate:
+// 1500-2000 cycles per round instead of 1170, 3.13 ms, now 2.29; 2.71, 2.43,
+// 2.29, 2.32 and 2.40 ms with 1, 2, 4, 8 and 32 first warps).
 __device__ __forceinline__ int ticket_allowance(unsigned long long head, unsigned long long tail,
                                                 bool waits)
 {
