@@ -95,8 +95,8 @@ struct DevField {
 };
 
 struct Header {  // at the start of the work space, 256 bytes
-    // The queue's hot words: atomics of every warp.  (tail, done) is read in
-    // one 16-byte access.
+    // The queue's hot words: atomics of every warp.  tail and done, side by
+    // side, are polled in one vector access.
     unsigned long long tail;      // slots reserved (stored or dropped)
     unsigned long long done;      // electrons finished or dropped
     unsigned long long head;      // next queue ticket
@@ -210,12 +210,20 @@ __device__ __forceinline__ unsigned int ld_relaxed_u32(const unsigned int *p)
     return v;
 }
 
-// Two neighbouring 64-bit words in one access of 16 bytes (16-byte aligned):
-// both as of the same moment.
+__device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p)
+{
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Two neighbouring 64-bit words (16-byte aligned) in one vector access: two
+// loads of no common moment.  (Not one 128-bit load: it would overlap the
+// words' 64-bit atomics in part, and the memory model promises nothing then.)
 __device__ __forceinline__ ulonglong2 ld_relaxed_u64x2(const unsigned long long *p)
 {
     ulonglong2 v;
-    asm volatile("{ .reg .b128 q; ld.relaxed.gpu.global.b128 q, [%2]; mov.b128 {%0, %1}, q; }"
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];"
                  : "=l"(v.x), "=l"(v.y) : "l"(p) : "memory");
     return v;
 }

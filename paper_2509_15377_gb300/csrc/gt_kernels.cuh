@@ -16,6 +16,7 @@
 #pragma once
 
 #include "gt_device.cuh"
+#include "gt_queue.h"
 
 namespace gt {
 
@@ -313,15 +314,14 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
             const bool waiting = !kShares || __any_sync(FULL, ticket >= 0);
             int verdict = 0;  // 0 wait, 1 finished, 2 give up
             if (lane == 0) {
-                // an electron's children are counted in tail before it is counted
-                // in done, so that equal counts of one moment mean the end
                 const ulonglong2 td = ld_relaxed_u64x2(&p.hdr->tail);
                 const unsigned err = ld_relaxed_u32(&p.hdr->error);
                 const unsigned long long tl = td.x, d = td.y;
                 if (kShares)
                     bs.allow[wid] = ticket_allowance(ld_relaxed_u64(&p.hdr->head), tl, !waiting);
                 const unsigned long long now = globaltimer();
-                if (d == tl) {
+                if (run_ended(tl, d, [&] { return ld_acquire_u64(&p.hdr->done); },
+                              [&] { return ld_acquire_u64(&p.hdr->tail); })) {
                     verdict = 1;
                 } else if (err & (ERR_TIMEOUT | ERR_BADARG)) {
                     verdict = 2;
