@@ -434,11 +434,11 @@ int gt_graph_destroy(gt_graph *graph);
  * their electron finishes).  gt_autotune runs `run` in GT_BATCHED mode (after
  * one warm-up run) and measures real collisions per millisecond of transport
  * kernel time (CUDA events) for the shapes of a coordinate descent: from a
- * middle shape, each dimension in turn takes its best value with the others
+ * middle shape (FP64: the default one), each dimension in turn takes its best value with the others
  * held, until a whole sweep changes nothing (at most four sweeps; a shape
  * runs at most once; typically 10-14 runs, so a sample large enough to keep
  * the GPU saturated is affordable).  Values: MIXED 512/768/896/1024 threads,
- * refill period 4/8/16/32, flights per phase 1/2/4/6; FP64 128/256/512
+ * refill period 4/8/16/32, flights per phase 1/2/4/6; FP64 128/160/256/512
  * threads, refill period 8/16/32/64.  A block, refill_period or
  * flights_per_phase set (non-zero) in `run` fixes that dimension.  The
  * fastest shape is remembered by the context for the run's
