@@ -180,12 +180,21 @@ typedef struct {
     uint32_t coll_limit;              /* real collisions per electron, 0: none */
     int32_t precision;                /* GT_FP64 / GT_MIXED */
     int32_t mode;                     /* GT_BATCHED / GT_PLAIN */
-    int32_t block;                    /* threads per CTA, 0 = default */
+    int32_t block;                    /* threads per CTA, a multiple of 32; 0 = the
+                                         shape of gt_autotune, else FP64 160, MIXED
+                                         512, or on a plate 768 to 1024 (banded
+                                         majorant, no B, no sub-steps) when the
+                                         capacity and the size expected from
+                                         primaries, gas and field promise a long
+                                         run and the gas table still fits */
     int32_t refill_period;            /* BATCHED: steps between refills of idle lanes
                                          from the queue (and FP32-to-FP64 flushes):
                                          FP64 one flight per step, MIXED one
                                          collision round per step; 0 = default */
-    int32_t grid;                     /* BATCHED: CTAs, 0 = one per SM */
+    int32_t grid;                     /* BATCHED: CTAs; 0 = as many as are resident
+                                         at once (one per SM with the default
+                                         block), in FP64 at most five warps per SM,
+                                         or one CTA if it has more */
     uint64_t size_limit;              /* BATCHED: max electrons per avalanche,
                                          further secondaries dropped; 0 = none */
     double spin_limit_ms;             /* longest wait without queue progress, 0 =

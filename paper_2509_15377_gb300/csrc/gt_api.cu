@@ -22,6 +22,7 @@ struct gt_ctx {
     int sms = 0;
     size_t smem_optin = 0;
     bool has_gas = false, has_field = false;
+    double ion_energy = -1.0, ion_field = 0.0;  // of the gas, see expected_electrons
     DevGas gas{};
     DevField field{};
     double *d_cum64 = nullptr;
@@ -167,17 +168,55 @@ Stack carve_stack(char *&p, int64_t cap)
 // 97 ms at 2 x 8 warps, 44.4 at 5; 46.9 at 4, 49.4 at 8, after the step itself became shorter).
 constexpr int kWarps64 = 5;
 
+// Electrons that a plate run may be expected to make, from what the host
+// knows of it (no capacity: a caller who does not know the gain reserves
+// generously): its primaries times the gain across the gap, with the Townsend
+// coefficient of noble gases, alpha = A exp(-B / sqrt(E)) (Ward, 1962).  By
+// its peak: alpha I / E is 0.25 at the field ion_field, where an electron gains
+// 0.29 I (I the lowest ionisation energy) in a mean free path at I.  For the
+// argon-like gas, from the oracle's gains: 0.003, 0.058, 0.146, 0.185, 0.209,
+// 0.227 and 0.244 at 5, 10, 20, 30, 40, 50 and 100 kV/cm, here 0.010, 0.052,
+// 0.135, 0.188, 0.218, 0.235 and 0.247.  A field per avalanche counts as e0;
+// how early a time or collision limit ends the growth is not estimated.
+double expected_electrons(const gt_ctx *ctx, const gt_run *r)
+{
+    const double e = ctx->field.e0, I = ctx->ion_energy;
+    double gain = 1.0;
+    if (I >= 0.0 && e > 0.0) {
+        const double y = std::sqrt(ctx->ion_field / e);
+        const double growth = 0.25 * y * y * std::exp(2.0 * (1.0 - y)) * e * ctx->field.gap / I;
+        gain = growth < 60.0 ? std::exp(growth) : 1e26;  // and where I = 0
+    }
+    double n = gain * (double)r->n_primaries;
+    if (r->size_limit) n = std::min(n, (double)r->size_limit * r->n_avalanches);
+    return n;
+}
+
 // Threads per CTA of a batched run that leaves them open.  Mixed: 512 (16 warps,
 // all the registers they want) has the shorter rounds, 1024 (64 registers, no
 // spills in the builds for the common run) the more electrons, and on a plate
-// it wins where the run is much longer than its longest chain: many primaries
-// and room for many electrons per lane of a full GPU.  At 512, 768, 896 and 1024:
-// 1000 avalanches of the 40 kV/cm plate (room for 11 per lane) 7.18, 7.15, 6.68
-// and 6.73 ms; 767 avalanches with three primaries and the general gas (50 per
-// lane) 21.6, 18.4, 16.6 and 16.1; exact crossings (11 per lane) 7.87, 7.18, 7.36
-// and 7.31; signals, whose state spills beyond 768, 18.5, 16.6, 16.7 and 17.8; 8
-// avalanches 2.27, 2.63, 3.7 and 3.7.  The global majorant's long chains and the
-// other fields' drifts stay at 512 (500 avalanches 17.0 at 512, 22.1 at 1024; the
+// it wins where the run is much longer than its longest chain: from about 7e5
+// electrons (4.5 per lane of a full GPU) on.  Plates at 512, 768, 896 and 1024
+// threads, in ms:
+//   40 kV/cm, 400 avalanches (3.9e5 electrons)    4.19   4.72   4.92   5.35
+//             600 (5.8e5)                         5.04   5.37   5.41   5.60
+//             800 (7.9e5)                         6.01   6.22   5.93   5.99
+//             1300 (1.3e6)                        8.60   8.39   7.78   7.72
+//   30 kV/cm, 400 (3.9e4)                         3.72   4.84   4.94   5.17
+//             2301 (2.2e5)                        4.39   5.59   5.74   6.21
+//             8000 (7.8e5)                        8.31   8.21   7.63   7.76
+//   general gas, 40 kV/cm, 2301 (2.5e6)          12.16  10.68   9.93   9.86
+//   exact crossings, 500 (4.9e5)                  4.65   4.64   5.12   5.41
+//             1300 (1.4e6)                        9.01   8.04   8.22   8.15
+//   signals (their state spills beyond 768),
+//             500 (5.0e5)                         4.93   5.03   5.61   6.67
+//             1300 (1.4e6)                        9.96   9.20   9.53  10.46
+// So the larger shapes want room for 8 electrons per lane (a run that is
+// reserved tightly has that from 8e5 electrons on) and 3 expected ones: the
+// estimate is good to a factor of 1.5 or so, and a run of that size loses
+// 5-15 % with either shape if it is the other's.  32 per lane for 1024 threads:
+// 896 are within 3 % there.  The global majorant's long chains and the other
+// fields' drifts stay at 512 (500 avalanches 17.0 at 512, 22.1 at 1024; the
 // 256^3 grid 112 and 154).
 int default_block(const gt_ctx *ctx, const gt_run *r, int64_t capacity)
 {
@@ -185,7 +224,8 @@ int default_block(const gt_ctx *ctx, const gt_run *r, int64_t capacity)
     const int64_t lanes = (int64_t)1024 * ctx->sms;
     if (r->mode != GT_BATCHED || r->majorant != GT_MAJORANT_BANDED ||
         ctx->field.kind != GT_FIELD_PLATE || ctx->field.has_b || r->substeps > 1 ||
-        r->n_primaries < 2 * ctx->sms || capacity < 8 * lanes)
+        r->n_primaries < 2 * ctx->sms || capacity < 8 * lanes ||
+        expected_electrons(ctx, r) < 3.0 * (double)lanes)
         return 512;
     if (r->signal_kind != GT_W_NONE && r->signal_bins > 0) return 768;
     if (capacity >= 32 * lanes) return 1024;
@@ -467,6 +507,24 @@ static int gas_table_upload_impl(gt_ctx *ctx, const gt_gas *g)
     d.any_special = d.any_aniso || g->split_w > 0.0;
     for (int j = 0; j < L; ++j)
         if (d.type[j] == GT_LEVEL_ATTACHMENT) d.any_special = 1;
+    // the lowest ionisation energy with a rate (-1: none) and the field of the
+    // largest ionisation per volt (expected_electrons)
+    ctx->ion_energy = -1.0;
+    ctx->ion_field = 0.0;
+    for (int j = 0; j < L; ++j) {
+        if (d.type[j] != GT_LEVEL_IONISATION) continue;
+        if (ctx->ion_energy >= 0.0 && d.thr[j] >= ctx->ion_energy) continue;
+        for (int k = 0; k < N; ++k)
+            if (g->rate[(size_t)k * L + j] > 0.0) {
+                ctx->ion_energy = d.thr[j];
+                break;
+            }
+    }
+    if (ctx->ion_energy > 0.0) {
+        const double I = ctx->ion_energy;
+        const size_t k = (size_t)std::min(I * d.inv_d_eps, N - 1.0);
+        ctx->ion_field = 0.29 * I * cum[k * L + L - 1] / std::sqrt(kTwoAccel * I);
+    }
     ctx->has_gas = true;
     ++ctx->setup_gen;
     return GT_OK;
