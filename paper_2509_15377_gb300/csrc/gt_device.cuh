@@ -1585,7 +1585,7 @@ struct Fp64Electron {
 //
 // Every rounding of the collision is written out (products fused or not as
 // stated): the warp's vote picks the straight-line or the general path, the
-// launch shape picks the build, and an electron's trajectory must not depend
+// threads per CTA pick the build, and an electron's trajectory must not depend
 // on either.  A build's own choice of fused products did: two builds of the
 // general gas gave different electrons, and so did two runs of the basic gas
 // with crossings or signals, where the two paths differed.
