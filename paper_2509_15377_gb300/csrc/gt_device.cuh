@@ -14,6 +14,7 @@
 #include <cuda_runtime.h>
 
 #include "gt_avalanche.h"
+#include "gt_math.h"
 
 namespace gt {
 
@@ -701,16 +702,6 @@ __device__ __forceinline__ void lorentz_step64(const DevField &f, double ax, dou
     vx = vp * bx + gx + ux * c - cx * s;
     vy = vp * by + gy + uy * c - cy * s;
     vz = vp * bz + gz + uz * c - cz * s;
-}
-
-// n / d, correctly rounded, for a divisor known in advance with r = 1/d
-// rounded: the first residual step makes the quotient faithful, the second
-// rounds it correctly (Markstein, IBM J. Res. Dev. 34, 111, 1990).
-__device__ __forceinline__ float div_known32(float n, float d, float r)
-{
-    float q = n * r;
-    q = fmaf(fmaf(-q, d, n), r, q);
-    return fmaf(fmaf(-q, d, n), r, q);
 }
 
 // a b + c d and a b - c d, the first product fused

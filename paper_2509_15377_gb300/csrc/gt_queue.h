@@ -2,11 +2,7 @@
 // compiler, which tries the decision on every pair of moments of its reads.
 #pragma once
 
-#ifdef __CUDACC__
-#define GT_HOST_DEVICE __host__ __device__ __forceinline__
-#else
-#define GT_HOST_DEVICE inline
-#endif
+#include "gt_math.h"
 
 namespace gt {
 
