@@ -1286,17 +1286,8 @@ static int avalanche_run_impl(gt_ctx *ctx, const gt_run *r, const gt_endpoints *
                 pa.n_active = n_active;
                 pa.parity = parity;
                 pa.aval = a;
-                // A generation lasts as long as its longest chain of flights: its
-                // electrons spread over the SMs first, then over up to four warps
-                // of each, then over the warps' lanes.  (128-thread blocks of 32
-                // electrons per warp put a generation of 100 on one SM, whose FP64
-                // pipe takes 16 clocks per warp instruction however many lanes are
-                // active: two avalanches of the 40 kV/cm plate 173 ms, now 112.)
-                const long long sms = ctx->sms;
-                const int warps = (int)std::min<long long>((n_active + sms - 1) / sms,
-                                                           std::min(block, 128) / 32);
-                const int pblock = 32 * warps;
-                pa.lanes = (int)std::min<long long>((n_active + sms * warps - 1) / (sms * warps), 32);
+                const int pblock = std::min(block, 128);
+                pa.split = plain_split(n_active, ctx->sms, pblock);
                 GT_CUDA(ctx, fp64 ? launch_plain_fp64(p, pa, pblock,
                                                       shared_bytes(L, ctx->gas.n_nodes, pblock, false, band_entries), s)
                                   : launch_plain_mixed(p, pa, smem_table, pblock,

@@ -16,6 +16,7 @@
 #pragma once
 
 #include "gt_device.cuh"
+#include "gt_plain.h"
 #include "gt_queue.h"
 
 namespace gt {
@@ -442,21 +443,20 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
 
 // One generation of one avalanche (plain mode): every electron of `cur`
 // flies until it ionises (it stays alive and its new electron goes to
-// `fresh`) or finishes (alive = 0).  Each warp holds `lanes` of them.
+// `fresh`) or finishes (alive = 0); plain_split places them.
 template <class E, int FK, bool SMEM_TABLE, int MAXT, bool PHYS = true, bool GEO = true>
 __global__ void __launch_bounds__(MAXT)
-    k_plain_transport(const RunParams p, const Stack cur, long long n_active, int lanes,
-                      const Stack fresh, int parity, int aval)
+    k_plain_transport(const RunParams p, const Stack cur, long long n_active,
+                      const PlainSplit split, const Stack fresh, int parity, int aval)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ BlockState bs;
     const Tables tb = stage_tables<SMEM_TABLE>(p, smem, bs);
     if (blockIdx.x == 0 && threadIdx.x == 0) p.hdr->n_next[parity] = 0ull;
     const unsigned long long t_start = p.hdr->t_start;
-    const int lane = threadIdx.x & 31;
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long i = warp * lanes + lane;
-    if (lane >= lanes || i >= n_active) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const long long i = ((long long)blockIdx.x * split.warps + wid) * split.lanes + lane;
+    if (wid >= split.warps || lane >= split.lanes || i >= n_active) return;
 
     E e;
     e.bind(tb);

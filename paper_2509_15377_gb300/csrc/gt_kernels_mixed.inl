@@ -120,8 +120,7 @@ static cudaError_t plain(const RunParams &p, const PlainArgs &a, int block, size
     const long long n = a.n_active;
     if (n <= 0) return cudaSuccess;
     k_plain_transport<MixedElectron, FK, TAB, kPlainThreadsMixed, PHYS, GEO>
-        <<<plain_blocks(a, block), block, smem, s>>>(p, a.cur, n, a.lanes, a.fresh, a.parity,
-                                                     a.aval);
+        <<<a.split.blocks, block, smem, s>>>(p, a.cur, n, a.split, a.fresh, a.parity, a.aval);
     return cudaGetLastError();
 }
 

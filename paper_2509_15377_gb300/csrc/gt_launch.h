@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "gt_device.cuh"
+#include "gt_plain.h"
 
 struct gt_ctx;
 
@@ -37,17 +38,10 @@ struct SeedArgs {
 struct PlainArgs {
     Stack cur, fresh, next;
     long long n_active;
-    int lanes;  // electrons per warp
+    PlainSplit split;
     int parity;
     int aval;
 };
-
-// Blocks of a plain generation: lanes electrons per warp.
-inline unsigned plain_blocks(const PlainArgs &a, int block)
-{
-    const long long per = (long long)a.lanes * (block / 32);
-    return (unsigned)((a.n_active + per - 1) / per);
-}
 
 // Per-precision transport launchers (gt_kernels_fp64.cu / gt_kernels_mixed.cu).
 // `smem_table` selects the shared-memory copy of the FP32 table.
