@@ -104,7 +104,8 @@ struct Header {  // at the start of the work space, 256 bytes
     unsigned long long pad0[13];
     // The rest in a 128-byte line of its own: every warp reads `error` once per
     // iteration, and beside the hot words that read waits for their atomics
-    // (4096 avalanches 87.4 -> 87.0 ms, the general gas 16.5 -> 16.1).
+    // (767 avalanches of the general gas 16.5 -> 16.1 ms; 4096 of the basic gas
+    // 87.4 and 87.0, within the noise).
     unsigned int error;           // ERR_* bits
     unsigned int pad1;
     unsigned long long dropped;   // secondaries not stored
@@ -676,7 +677,8 @@ __device__ __forceinline__ int boundary64(const DevField &f, double x, double y,
 // |w|, w-hat and the reciprocals are the field's (field_setup): the step was
 // bound by the latency of its eight divisions and three square roots, seven
 // of them the same for every flight (a lone electron's round in the tube
-// with 1 T: 3215 cycles, now 1830; the 512-avalanche run 222 ms, now 140).
+// with 1 T: 3215 cycles -> 1830; the transport of 512 avalanches 222 -> 141 ms,
+// and 119-133 with the tube's own build for B).
 __device__ __forceinline__ void lorentz_step64(const DevField &f, double ax, double ay, double az,
                                                double dt, double &vx, double &vy, double &vz,
                                                double &dx, double &dy, double &dz)
@@ -826,7 +828,8 @@ __device__ __forceinline__ int select_below_total32(const float *c0, int stride,
 // Band of an energy: floor(eps / band width), clamped to the band range.
 __device__ __forceinline__ int band_index64(const DevGas &g, double eps)
 {
-    // the conversion truncates, saturates and takes a NaN to 0
+    // the conversion truncates and saturates; a NaN comes out as INT_MIN, which
+    // the max() takes to band 0
     return max(min(__double2int_rz(eps * g.inv_band_width), g.n_bands - 1), 0);
 }
 
@@ -1997,7 +2000,7 @@ struct MixedElectron {
     // the sub-steps and exact crossings of fly_steps().
     // MAJ = kMajBandedB builds the step of MAJ = 1 for runs in a magnetic field
     // (512 avalanches in the tube with 1 T: a lone electron 1894 cycles per
-    // flight, now 1576; 143 -> 126 ms).
+    // flight, now 1576; transport 141 -> 119-133 ms).
     // MAJ = kMajGlobal builds the step for runs with the global majorant and
     // no magnetic field, without the branches of the others (500
     // avalanches of the 40 kV/cm plate 17.1 -> 16.4 ms).

@@ -295,8 +295,9 @@ __global__ void __launch_bounds__(MAXT) k_batched(const RunParams p)
                 has = true;
                 // a new electron starts where its parent's boundary test has just
                 // found it inside; only a primary's start is tested (on a mesh the
-                // test scans a bin of elements in FP64: it took two thirds of the
-                // 48-avalanche mesh run, 195 ms, now 52)
+                // test scans a bin of elements in FP64: the transport of 48
+                // avalanches took 195 ms with it and 52 without; 41 with the
+                // later changes to the mesh)
                 if (e.slot < p.n_primaries && (e.template check_start<FK>(p) & EV_RETIRE)) {
                     finish<GEO>(p, tb, e, bs);
                     has = false;
